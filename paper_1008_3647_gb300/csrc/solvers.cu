@@ -1212,7 +1212,10 @@ ufg_status two_step(ufg_solver* S, ufg_field* f, const double* b, double* x, boo
     return UFG_OK;
   }
   UFG_TRY(solve_system(S, f, OPK_MDAG, b, S->y64, false, 0.5 * tol, p, o1));
-  if (o1->done != 1) return UFG_OK;
+  if (o1->done != 1) {  // no second step: x is the initial guess
+    if (!x0) UFG_CUDA(cudaMemsetAsync(x, 0, S->lat->S * sizeof(double), S->st));
+    return UFG_OK;
+  }
   UFG_TRY(norm64(S, S->y64, S->lat->S, &yn));
   const double tol2 = tol * bn / (2.0 * (2.0 + S->lat->A) * yn);
   UFG_TRY(solve_system(S, f, OPK_M, S->y64, x, x0, tol2, p, o2));

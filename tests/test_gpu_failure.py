@@ -132,3 +132,16 @@ def test_force_finishes_a_broken_down_solve_with_cg(ufg):
     # (1e-11: this unpreconditioned solution spans a wide range, so the force entries do too)
     assert float(np.abs(dS.cpu().numpy() - ref).max() / np.abs(ref).max()) < 1e-11
     assert S == pytest.approx(float(np.dot(b.ravel(), Xh.ravel())), rel=1e-12)
+
+
+def test_broken_down_first_step_leaves_no_garbage_in_x(ufg):
+    # the second step never runs, so x is the initial guess: zero without one
+    nx, ntau = 8, 64
+    sigma, b = field_and_source(nx, ntau, 0)
+    lat = ufg.Lattice(nx, ntau)
+    field = ufg.Field(lat, torch.from_numpy(sigma).cuda())
+    solver = ufg.Solver(lat)
+    x = torch.full(lat.shape, float("nan"), dtype=torch.float64, device="cuda")
+    x, st = solver.ufg_solve_bicgstab_two_step(field, torch.from_numpy(b).cuda(), x, tol=1e-10)
+    assert st["status"] == ufg.UFG_BREAKDOWN and st["iterations_step"][1] == 0
+    assert bool((x == 0).all())
