@@ -34,7 +34,7 @@
  *   UFG_PDL=1          every kernel is launched with programmatic dependent launch (by
  *                      default only the launches of the standalone operator calls below);
  *   UFG_NO_FUSED_Q=1   Q = M^T M as two launches (M, then M^T) everywhere (by default one
- *                      kernel per output slice on 16^3 lattices with N_tau <= twice the SMs);
+ *                      kernel per output slice on FP32 16^3 lattices, N_tau <= twice the SMs);
  *   UFG_NO_MOMENTUM=1  WCE-preconditioned BiCGStab stays in the position basis (by default it
  *                      iterates on F x where the lattice has the fused momentum-space operator);
  *   UFG_NO_PAIR=1      FP32 16^3 slices run one line per thread instead of two (packed FP32x2);
@@ -61,13 +61,9 @@ typedef enum {
   UFG_UNSUPPORTED = 9    /* valid input outside what the library implements (e.g. N_x) */
 } ufg_status;
 
-/* UFG_FP64_EMULATED: FP64 vectors, arithmetic in double-float pairs on the FP32 pipe (about 46
- * significant bits; GB300's FP64 pipe is ~1/76 of its FP32 rate).  Accepted by
- * ufg_apply_M_momentum.  Its absolute error is about 2^-46 ||M|| ||x||, so a residual b - M x of
- * a nearly converged, ill-conditioned system (||x|| >> ||b||) is not resolved to 1e-10 of
- * ||b|| this way.  The batched mixed-precision solve uses it only for incremental residual
- * updates r -= M d after a first FP64 residual, where the error scales with the increment d;
- * every final residual is FP64. */
+/* UFG_FP64_EMULATED: FP64 vectors, accepted by ufg_apply_M_momentum for the operator without
+ * FP64 arithmetic in its line passes.  UFG_FP64 runs those on the integer pipe too, so the two
+ * are the same kernel. */
 typedef enum { UFG_FP64 = 0, UFG_FP32 = 1, UFG_MIXED = 2, UFG_FP64_EMULATED = 3 } ufg_precision;
 
 /* UFG_PC_SCA_CHEB: the strong-coupling factorisation with the Chebyshev polynomial as a secondary
@@ -250,8 +246,8 @@ double ufg_lattice_coupling(const ufg_lattice* lat);
  * message) if any kernel launched on the lattice since the last check ran out of its wait, else
  * UFG_OK.  The paper has no counterpart (failure reporting of this library). */
 ufg_status ufg_lattice_check(const ufg_lattice* lat, void* stream);
-/* Test hook for the failure path above: the next `launches` TMA-staged slice-kernel launches (in
- * any lattice of the process) each run one extra bounded wait on a barrier whose expected bytes
+/* Test hook for the failure path above: the next `launches` TMA-staged FP32 or FP64 N_x = 8, 16
+ * slice-kernel launches (in any lattice of the process) each run one extra bounded wait on a barrier whose expected bytes
  * never arrive, so that wait runs out after a few hundred polling rounds and raises the flag
  * exactly as a real timeout would.  The kernel's own copies complete as usual, nothing faults or
  * hangs, and the results stay correct; only the reported status changes.  0 cancels. */
@@ -283,7 +279,7 @@ void ufg_field_destroy(ufg_field* f);
  * [1 - exp(-i omega - tau E(k))]^{-1} in frequency-momentum space, omega = (2n+1) pi / N_tau).
  * precision UFG_FP64: x, y are double*; UFG_FP32: float*.  x and y must not overlap.  Q and
  * M0^{-1}/M0^{-T} use library workspace of the field, so calls on one field must not overlap in
- * time on different streams.  Q on a 16^3 lattice with 3 <= N_tau <= twice the GPU's SM count
+ * time on different streams.  FP32 Q on a 16^3 lattice with 3 <= N_tau <= twice the GPU's SM count
  * runs as one kernel per output slice (x at t-1, t, t+1 in shared memory, three kinetic
  * stages, no intermediate vector); elsewhere as M followed by M^T. */
 ufg_status ufg_apply_M(ufg_field* f, const void* x, void* y, int precision, void* stream);
@@ -304,7 +300,7 @@ ufg_status ufg_apply_M0invT(ufg_field* f, const void* x, void* y, int precision,
  * fused kernel per slice (inverse transform, site multiplier, forward transform, the M0 part of
  * Sec. 3 and the identity).  Built for FP32 N_x = 16 and FP64 N_x = 8, 16; UFG_INVALID_ARG
  * elsewhere.  Same precision, alignment and overlap rules as the applies above; precision
- * UFG_FP64_EMULATED also takes FP64 vectors (double-float arithmetic). */
+ * UFG_FP64_EMULATED also takes FP64 vectors. */
 ufg_status ufg_fourier(ufg_field* f, const void* x, void* y, int precision, int inverse,
                        void* stream);
 ufg_status ufg_apply_M_momentum(ufg_field* f, const void* x, void* y, int precision,

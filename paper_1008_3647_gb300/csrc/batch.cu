@@ -159,15 +159,13 @@ ufg_status slice(Batch& B, Group& g, SliceCall c, int exec_if) {
 
 // out = a * (A in) + bU * U with partials (out.dotP, out.out), all groups; fop >= 0 applies that
 // scalar op to each problem from the partials in the same launch
-// emulate64 (FP64, momentum basis): double-float arithmetic on the FP32 pipe (slice_df.cuh)
 ufg_status apply_b(Batch& B, int prec, int op, const void* in, void* out, double a, const void* U,
                    double bU, const void* dotP, bool self, double* part, int exec_if,
-                   int fop = -1, bool emulate64 = false) {
+                   int fop = -1) {
   if (B.mom) {  // the fused momentum-space operator, one kernel per group
     for (auto& g : B.groups) {
       SliceCall c = base_call(g.lat, FAM_INV, prec);
       c.fam = FAM_M1W;
-      c.emulate64 = (emulate64 && prec == 0) ? 1 : 0;
       c.coef2 = base_call(g.lat, FAM_FWD, prec).coef;
       c.m1w_full = 1;
       c.in = in;
@@ -668,10 +666,9 @@ ufg_status solve_in_basis(Batch& B, int op, const double* rhs, double* x,
   constexpr int RU_SPAN = 60;
   // Incremental reliable updates (momentum basis): after a problem's first update r holds its
   // FP64 true residual, and a later update x += d (d = ||rhs|| x32) needs only
-  // r -= A d, computed by the double-float operator (slice_df.cuh) on the FP32 pipe.  Its error,
-  // about 2^-46 ||A|| ||d||, scales with the increment (||d|| ~ ||A^-1|| ||r||), not with x,
+  // r -= A d: its rounding error scales with the increment (||d|| ~ ||A^-1|| ||r||), not with x,
   // so it stays far below the residual it corrects; the first update of each solve and the
-  // final residual of every problem are FP64.
+  // final residual of every problem are taken from x.
   constexpr int RU_INC = 8;  // solver flag of the problems inside an incremental update
   std::vector<char> have_r(B.n, 0);
   std::vector<char> fallback(B.n, 0), verified(B.n, 0);
@@ -748,12 +745,11 @@ ufg_status solve_in_basis(Batch& B, int op, const double* rhs, double* x,
     }
     UFG_TRY(mixed_glue(B, 2, x, (float*)V.x, sc_full, &sc_inc, B.d64));
     UFG_TRY(write_scs(B));
-    // true residual: r = rhs - A x in FP64, or r -= A d in double-float arithmetic
+    // true residual: r = rhs - A x, or r -= A d
     if (any_full)
       UFG_TRY(apply_b(B, 0, op, x, B.r64, -1.0, rhs, 1.0, nullptr, false, nullptr, RU_BUSY));
     if (any_inc)
-      UFG_TRY(apply_b(B, 0, op, B.d64, B.r64, -1.0, B.r64, 1.0, nullptr, false, nullptr, RU_INC,
-                      -1, true));
+      UFG_TRY(apply_b(B, 0, op, B.d64, B.r64, -1.0, B.r64, 1.0, nullptr, false, nullptr, RU_INC));
     UFG_TRY(norms_b(B, B.r64, rn));  // reads the scalars back
     std::vector<double> inv2(B.n, 0.0);
     bool cont = false;
@@ -915,11 +911,13 @@ ufg_status build_slice_tiles(Batch& B, const ufg_problem* probs) {
 }
 
 // Time slices per slice tile, tuned per (N_x, tau) group whose slice kernels are the
-// shared-memory ones in both precisions (no TMA shape at this N_x; the TMA kernels take one
-// slice per CTA): at N_x = 6 a one-slice tile keeps 36 of 256 threads busy in a pass.  Each
-// candidate (1, 2, 4, 8 slices within 48 KB of FP64 shared memory and the group's longest
-// N_tau) is timed on the batch's own arenas with the M apply in both precisions (zeroed
-// operands, three launches each after one), and the fastest is kept (ufg_stats.tile_slices).
+// shared-memory ones in FP32 (no TMA shape at this N_x; the TMA kernels take one slice per CTA):
+// at N_x = 6 a one-slice tile keeps 36 of 256 threads busy in a pass.  Each candidate (1, 2, 4, 8
+// slices within 48 KB of FP64 shared memory and the group's longest N_tau) is timed on the
+// batch's own arenas with the FP32 M apply, where mixed solves spend their time (with the FP64
+// apply in the sum the 96-problem batch chose one slice at N_x = 10 and 12 and took 78.9 instead
+// of 74.5 ms), on zeroed operands, three launches each after one; the fastest is kept
+// (ufg_stats.tile_slices).
 ufg_status tune_tiles(Batch& B, const ufg_problem* probs) {
   auto tma_shape = [](int N, int prec) { return prec ? (N == 16 || N == 32) : (N == 8 || N == 16); };
   bool changed = false, zeroed = false;
@@ -938,15 +936,10 @@ ufg_status tune_tiles(Batch& B, const ufg_problem* probs) {
     }
     if (cand.size() < 2) continue;
     if (!zeroed) {
-      const size_t S = (size_t)B.S;
-      for (int prec = 0; prec < 2; ++prec) {
-        const size_t es = prec ? sizeof(float) : sizeof(double);
-        if (cudaMemsetAsync(B.ar[prec].x, 0, S * es, B.st) != cudaSuccess ||
-            cudaMemsetAsync(const_cast<void*>(fldb(B, 'w', prec)), 0, S * es, B.st) !=
-                cudaSuccess) {
-          result = cuda_fail(cudaGetLastError(), "tile tuning");
-          break;
-        }
+      if (cudaMemsetAsync(B.ar[1].x, 0, (size_t)B.S * sizeof(float), B.st) != cudaSuccess ||
+          cudaMemsetAsync(B.w32, 0, (size_t)B.S * sizeof(float), B.st) != cudaSuccess) {
+        result = cuda_fail(cudaGetLastError(), "tile tuning");
+        break;
       }
       zeroed = true;
     }
@@ -955,29 +948,23 @@ ufg_status tune_tiles(Batch& B, const ufg_problem* probs) {
     for (int spc : cand) {
       g.spc = spc;
       if ((result = build_slice_tiles(B, probs)) != UFG_OK) break;
-      float total = 0.0f;
-      for (int prec = 0; prec < 2 && result == UFG_OK; ++prec) {
-        SliceCall c = base_call(g.lat, FAM_KIN, prec);
-        c.in = B.ar[prec].x;
-        c.pre = fldb(B, 'w', prec);
-        c.id = c.in;
-        c.shift = -1;
-        c.out = B.ar[prec].t;
-        if ((result = slice(B, g, c, -1)) != UFG_OK) break;  // warm-up
-        cudaEventRecord(e0, B.st);
-        for (int r = 0; r < 3 && result == UFG_OK; ++r) result = slice(B, g, c, -1);
-        cudaEventRecord(e1, B.st);
-        if (cudaEventSynchronize(e1) != cudaSuccess) {
-          result = cuda_fail(cudaGetLastError(), "tile tuning");
-          break;
-        }
-        float ms = 0.0f;
-        cudaEventElapsedTime(&ms, e0, e1);
-        total += ms;
-      }
+      SliceCall c = base_call(g.lat, FAM_KIN, 1);
+      c.in = B.ar[1].x;
+      c.pre = B.w32;
+      c.id = c.in;
+      c.shift = -1;
+      c.out = B.ar[1].t;
+      if ((result = slice(B, g, c, -1)) != UFG_OK) break;  // warm-up
+      cudaEventRecord(e0, B.st);
+      for (int r = 0; r < 3 && result == UFG_OK; ++r) result = slice(B, g, c, -1);
+      cudaEventRecord(e1, B.st);
+      if (result == UFG_OK && cudaEventSynchronize(e1) != cudaSuccess)
+        result = cuda_fail(cudaGetLastError(), "tile tuning");
       if (result != UFG_OK) break;
-      if (total < best) {
-        best = total;
+      float ms = 0.0f;
+      cudaEventElapsedTime(&ms, e0, e1);
+      if (ms < best) {
+        best = ms;
         best_spc = spc;
       }
     }

@@ -23,11 +23,10 @@ bool slice_q_supported(int N, int prec, int ntau, int dim) {
     const char* t = std::getenv("UFG_NO_TMA");
     env = ((e && e[0] == '1') || (t && t[0] == '1')) ? 0 : 1;
   }
-  if (!env || dim != 3 || N != 16 || ntau < 3) return false;
+  if (!env || dim != 3 || N != 16 || prec != 1 || ntau < 3) return false;
   // one CTA per output slice with three kinetic stages: ahead of the two launches of M and M^T
-  // while their slices fill at most about two CTAs per SM (16^3 x 256: 10.6 against 13.4 us in
-  // FP32, 183 against 191 us in FP64); behind them on longer lattices (16^3 x 1024 FP32: 23.0
-  // against 19.1 us) and on 8^3 slices (FP64 8^3 x 64: 17.3 against 14.7 us)
+  // while their slices fill at most about two CTAs per SM (16^3 x 256: 10.6 against 13.4 us);
+  // behind them on longer lattices (16^3 x 1024: 23.0 against 19.1 us)
   static int sms = 0;
   if (sms == 0) {
     int dev = 0, v = 0;
@@ -36,7 +35,6 @@ bool slice_q_supported(int N, int prec, int ntau, int dim) {
       v = 152;
     sms = v;
   }
-  (void)prec;
   return ntau <= 2 * sms;
 }
 

@@ -10,7 +10,7 @@
 #include <vector>
 
 #include "launch.cuh"
-#include "line_ops.cuh"
+#include "fix_ops.cuh"
 #include "ufg_internal.h"
 
 namespace ufg {
@@ -264,6 +264,27 @@ static void pack(const std::vector<double>& flat, std::vector<unsigned char>& ou
   std::memcpy(out.data(), v.data(), out.size());
 }
 
+template <int N>
+static bool pack_fix_n(const double* flat, std::vector<unsigned char>& out) {
+  LineCoefFix<N> t;
+  if (!fix_table<N>(flat, &t)) return false;
+  out.resize(sizeof(t));
+  std::memcpy(out.data(), &t, sizeof(t));
+  return true;
+}
+static bool pack_fix(int N, const double* flat, std::vector<unsigned char>& out) {
+  switch (N) {
+    case 4: return pack_fix_n<4>(flat, out);
+    case 6: return pack_fix_n<6>(flat, out);
+    case 8: return pack_fix_n<8>(flat, out);
+    case 10: return pack_fix_n<10>(flat, out);
+    case 12: return pack_fix_n<12>(flat, out);
+    case 16: return pack_fix_n<16>(flat, out);
+    case 32: return pack_fix_n<32>(flat, out);
+  }
+  return false;
+}
+
 static ufg_status build_tables(ufg_lattice* L) {
   const int N = L->nx, H = N / 2;
   const double pi = 3.14159265358979323846;
@@ -297,6 +318,10 @@ static ufg_status build_tables(ufg_lattice* L) {
       return UFG_INTERNAL;
     }
     pack<double>(flat, L->coef[sp.fam][0]);
+    if (!pack_fix(N, flat.data(), L->coef_fix[sp.fam])) {
+      set_error("line operator of family %d exceeds the fixed-point range", sp.fam);
+      return UFG_INTERNAL;
+    }
     pack<float>(flat, L->coef[sp.fam][1]);
   }
   // per-mode table in spectral layout [sz][sy][sx] (dim 3; [sy][sx], [sx] below): the product
@@ -341,13 +366,30 @@ SliceCall base_call(const ufg_lattice* lat, int fam, int prec) {
   SliceCall c;
   c.fam = fam;
   c.prec = prec;
-  c.coef = lat->coef[fam][prec].data();
+  // FP64 on 3-D lattices runs on the integer pipe and takes the fixed-point tables
+  c.coef = prec == 0 && lat->dim == 3 ? lat->coef_fix[fam].data() : lat->coef[fam][prec].data();
   c.ntau = lat->ntau;
   c.dim = lat->dim;
   c.spc = lat->spc[prec];
   c.C = lat->C[prec];
   c.err = lat->dev_err;
   c.allow_tma = lat->use_tma[prec];
+  return c;
+}
+
+// FP64 kinetic calls on a 32^3 lattice with the line passes on the FP64 pipe.  A mixed-precision
+// solution at 1e-10 of an HMC right-hand side phi = M^T eta is determined to about 1e-7 only, and
+// any other rounding of phi or of the solve's FP64 residuals moves it by as much; M^T and those
+// residuals therefore keep the arithmetic that such solutions were made with.  1.49 ms a call at
+// 32^3 x 512, against 0.36 ms on the integer pipe, which every other FP64 call takes.
+SliceCall base_call_fp64(const ufg_lattice* lat) {
+  SliceCall c = base_call(lat, FAM_KIN, 0);
+  if (lat->dim == 3 && lat->nx == 32) {
+    c.fp64_pipe = 1;
+    c.coef = lat->coef[FAM_KIN][0].data();
+    c.C = 4;
+    c.spc = 1;
+  }
   return c;
 }
 
@@ -377,8 +419,9 @@ ufg_status op_M(const ufg_field* f, int prec, const void* x, void* y, cudaStream
   return run(f->lat, c, st);
 }
 
-ufg_status op_Mdag(const ufg_field* f, int prec, const void* x, void* y, cudaStream_t st) {
-  SliceCall c = base_call(f->lat, FAM_KIN, prec);
+ufg_status op_Mdag(const ufg_field* f, int prec, const void* x, void* y, cudaStream_t st,
+                   bool fp64_pipe) {
+  SliceCall c = fp64_pipe && prec == 0 ? base_call_fp64(f->lat) : base_call(f->lat, FAM_KIN, prec);
   c.in = x;
   c.post = fld(f, 'w', prec);
   c.id = x;
@@ -608,7 +651,7 @@ ufg_status ufg_apply_Mdag(ufg_field* f, const void* x, void* y, int prec, void* 
   clear_error();
   PdlScope pdl;
   UFG_TRY(check_vec(f, x, y, prec));
-  return op_Mdag(f, prec, x, y, as_stream(stream));
+  return op_Mdag(f, prec, x, y, as_stream(stream), true);
 }
 
 ufg_status ufg_apply_Q(ufg_field* f, const void* x, void* y, int prec, void* stream) {
@@ -693,8 +736,7 @@ ufg_status ufg_apply_M_momentum(ufg_field* f, const void* x, void* y, int prec, 
                                 void* stream) {
   clear_error();
   PdlScope pdl;
-  const bool emulated = (prec == UFG_FP64_EMULATED);
-  if (emulated) prec = UFG_FP64;
+  if (prec == UFG_FP64_EMULATED) prec = UFG_FP64;
   UFG_TRY(check_vec(f, x, y, prec));
   const ufg_lattice* lat = f->lat;
   if (lat->dim != 3 || !slice_m1w_supported(lat->nx, prec)) {
@@ -714,7 +756,6 @@ ufg_status ufg_apply_M_momentum(ufg_field* f, const void* x, void* y, int prec, 
   c.shift = transpose ? +1 : -1;
   c.a = 1.0;
   c.out = y;
-  c.emulate64 = emulated ? 1 : 0;
   return run(lat, c, as_stream(stream));
 }
 
@@ -815,7 +856,7 @@ extern "C" ufg_status ufg_lattice_autotune(ufg_lattice* L, void* stream) {
     const size_t es = prec ? 4 : 8;
     const int cs[] = {1, 2, 4};
     for (int c : cs) {
-      if (c > 1 && N < 16) continue;
+      if (c > 1 && (N < 16 || prec == 0)) continue;  // FP64: only the slices per CTA vary
       if (N % c) continue;
       for (int s = 1; s <= 8; s *= 2) {
         const size_t smem = (size_t)s * (N / c) * N * (N + 1) * es;

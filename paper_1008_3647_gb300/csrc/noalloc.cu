@@ -12,7 +12,7 @@
 #include <mutex>
 #include <vector>
 
-#include "line_ops.cuh"
+#include "fix_ops.cuh"
 #include "ufg_internal.h"
 #include "launch.cuh"
 
@@ -67,7 +67,7 @@ __global__ void noalloc_w_kernel(const double* __restrict__ sigma, double A, lon
 //   co[i][j] = (T[i-j] - T[i+j]) / 2   (indices mod N),
 // split further into the kernel's coefficient layout (host memory only).
 template <int N>
-bool kinetic_coef(double tau, int dispersion, LineCoef<N, double>* c) {
+bool kinetic_coef(double tau, int dispersion, LineCoefFix<N>* c) {
   constexpr int H = N / 2;
   const double pi = 3.14159265358979323846;
   double T[N];
@@ -90,14 +90,13 @@ bool kinetic_coef(double tau, int dispersion, LineCoef<N, double>* c) {
     for (int j = 1; j < H; ++j) co[(i - 1) * (H - 1) + (j - 1)] = 0.5 * (t(i - j) - t(i + j));
   if (!line_coef_flat(N, ce, co, false, false, flat) || (int)flat.size() != LineShape<N>::NC)
     return false;
-  for (int i = 0; i < LineShape<N>::NC; ++i) c->c[i] = flat[i];
-  return true;
+  return fix_table<N>(flat.data(), c);
 }
 
 template <int N>
 ufg_status run_q(int ntau, double tau, int dispersion, double A, const double* x, double* y,
                  double* w, double* t, cudaStream_t st) {
-  LineCoef<N, double> coef;
+  LineCoefFix<N> coef;
   if (!kinetic_coef<N>(tau, dispersion, &coef)) {
     set_error("apply_Q_noalloc: kinetic line operator does not split");
     return UFG_INTERNAL;

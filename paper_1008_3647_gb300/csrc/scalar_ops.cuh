@@ -175,4 +175,45 @@ static __device__ __forceinline__ void last_block_update(int op, DevScalars* sc,
   }
 }
 
+// last_block_update for CTAs of any whole number of warps (the FP64 slice kernels, whose CTA size
+// follows the lattice extent).
+static __device__ __forceinline__ void last_block_update_any(int op, DevScalars* sc,
+                                                            const double* part, int i0, int i1,
+                                                            unsigned* counter) {
+  __shared__ int is_last;
+  __shared__ double red[32][2];
+  const int tid = threadIdx.x, nw = (int)(blockDim.x >> 5);
+  if (tid == 0) {
+    __threadfence();
+    is_last = atomicAdd(counter, 1u) == (unsigned)(i1 - i0 - 1);
+  }
+  __syncthreads();
+  if (!is_last) return;
+  __threadfence();
+  double s0 = 0.0, s1 = 0.0;
+  for (int i = i0 + tid; i < i1; i += (int)blockDim.x) {
+    s0 += part[2 * i];
+    s1 += part[2 * i + 1];
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    s0 += __shfl_xor_sync(0xffffffffu, s0, off);
+    s1 += __shfl_xor_sync(0xffffffffu, s1, off);
+  }
+  if ((tid & 31) == 0) {
+    red[tid >> 5][0] = s0;
+    red[tid >> 5][1] = s1;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    s0 = s1 = 0.0;
+    for (int w = 0; w < nw; ++w) {
+      s0 += red[w][0];
+      s1 += red[w][1];
+    }
+    scalar_update(op, sc, part, s0, s1, nullptr, 0.0, 0.0);
+    *counter = 0u;
+  }
+}
+
 }  // namespace ufg

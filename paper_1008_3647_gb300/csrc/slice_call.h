@@ -83,11 +83,10 @@ struct SliceCall {
   // basis, out = full_scale * M x + bU * U with the partials as the KIN family; pre is then the
   // potential w = 1 + A sin(sigma) and a = 1
   int m1w_full = 0;
+  // FP64 on 32^3 lattices: the line passes on the FP64 pipe (slice_kernel.cuh) instead of the
+  // integer pipe, with `coef` the FP64 table (base_call_fp64)
+  int fp64_pipe = 0;
   double full_scale = 1.0;
-  // FAM_M1W FULL on FP64 vectors: double-float arithmetic on the FP32 pipe (slice_df.cuh) instead
-  // of FP64 arithmetic (ufg_apply_M_momentum with UFG_FP64_EMULATED; the batched incremental
-  // reliable updates)
-  int emulate64 = 0;
 };
 
 // Test hook of ufg_test_expire_waits: 1 if this TMA launch on st runs one bounded wait that is

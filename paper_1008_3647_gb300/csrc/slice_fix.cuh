@@ -1,0 +1,601 @@
+// FP64 slice kernels on the integer pipe (fix_ops.cuh): the line passes of every FP64 apply,
+// transform and fused momentum-space operator on 3-D lattices.
+//
+// A warp owns PW whole z-planes of one output slice, lanes = (plane p, column x), so the y-pass
+// takes its lines straight from global memory (consecutive x: full sectors, no staging), the x-
+// and y-passes exchange through the warp's own planes of shared memory with no CTA barrier, and
+// the warp's lines share one exponent (a tile).  Between passes the slice stays in 64-bit
+// integers; only the z-pass, whose lines cross the warps, aligns the tiles' exponents, and only
+// the epilogue converts back.  For the z-pass lanes = (row r, column x) with PW whole y-rows per
+// warp, so its loads, stores and epilogue operands are consecutive in x as well.
+//
+//   CTA = spc slices x TS threads (TS = 32 per PW planes), one line per thread and pass, no loops
+//   around a pass (the compiler moves the coefficients out of them into registers, 4 KB of
+//   spills at N = 32); padded rows of N + 1 words keep every exchange free of bank conflicts.
+//   N = 32: a cluster of 8 CTAs of 128 threads holds one slice, four planes each; the z-pass
+//   reads the other CTAs' planes through distributed shared memory.
+//
+// Bound by the ALU pipe (16^3 x 1024: 56 % busy, FP64 pipe 36 %, 24 warps per SM) and, at N = 32,
+// by instruction fetch (12 warps per SM, straight-line passes of 33 KB).  us per call, FP64-pipe
+// kernels before -> now: M 32^3 x 512 1473 -> 357, 16^3 x 1024 218 -> 42, 16^3 x 256 93 -> 19,
+// 12^3 x 120 32 -> 11; momentum-space M 16^3 x 1024 353 -> 91 (double-float 247).  Tried: one loop
+// over the three passes with the table indexed by the pass (688 us at 32^3, 57 at 16^3: the
+// coefficients come through LDC), the table in shared memory (706, 55: a broadcast moves 4 bytes a
+// cycle).
+#pragma once
+#include <cooperative_groups.h>
+#include <cuda_runtime.h>
+
+#include <cstring>
+
+#include "fix_ops.cuh"
+#include "launch.cuh"
+#include "mbarrier.cuh"
+#include "scalar_ops.cuh"
+#include "slice_call.h"
+#include "slice_kernel.cuh"
+
+namespace ufg {
+
+template <int N>
+struct FixShape {
+  static constexpr int C = N >= 32 ? 8 : 1;  // CTAs per slice
+  // planes (rows) per warp: the largest divisor of N with PW N <= 32
+  static constexpr int PW = N == 4 ? 4 : N == 6 ? 3 : N == 8 ? 4 : N == 32 ? 1 : 2;
+  static_assert(N % PW == 0 && N * PW <= 32, "a warp holds whole planes");
+  static constexpr int NPC = N / C;     // planes per CTA and slice
+  static constexpr int WPS = NPC / PW;  // warps per CTA and slice
+  static constexpr int TS = 32 * WPS;
+  static constexpr int P = N + 1;
+  static constexpr int PL = N * P;
+  // 64-bit words per CTA and slice
+  static constexpr int SLOT = NPC * PL;
+  static constexpr int NTILE = N / PW;   // tiles of one slice
+  // slices per CTA that the launchers may ask for (lattice and batch tile shapes)
+  static constexpr int MAXS = N == 4 ? 8 : N == 6 ? 8 : N == 8 ? 4 : N == 10 ? 4 : N == 12 ? 2 : 1;
+  static constexpr int NT = TS * MAXS;
+};
+
+template <int N>
+struct FixArgs {
+  LineCoefFix<N> cf[3];  // one copy per pass
+  const double* in;
+  const double* pre;
+  const double* bkpre;
+  const double* bkpost;
+  double* out;
+  const double* id;
+  const double* post;
+  const double* post2;
+  const double* U;
+  const double* V;
+  const double* dotP;
+  double a, bU, cV;
+  double* partials;
+  int want_dotP, want_self;
+  const int* done;
+  int exec_if;
+  const BatchTile* tiles;
+  const BatchProb* probs;
+  int scale_by_A;
+  int ntau, shift, spc;
+  int fop;
+  DevScalars* scs;
+  unsigned* counters;
+  int part_base;
+  int* err;
+  int expire;  // test hook (ufg_test_expire_waits)
+};
+
+// The thread's place in a work unit.
+template <int N>
+struct FixPos {
+  int s, wl, lane, lp, lx, line;  // slice, warp, lane; (plane or row, column); line = wl PW + lp
+  bool on;
+};
+template <int N>
+__device__ __forceinline__ FixPos<N> fix_pos() {
+  using S = FixShape<N>;
+  FixPos<N> p;
+  const int tid = threadIdx.x;
+  p.s = tid / S::TS;
+  const int ts = tid - p.s * S::TS;
+  p.wl = ts >> 5;
+  p.lane = ts & 31;
+  p.lp = p.lane / N;
+  p.lx = p.lane - p.lp * N;
+  p.line = p.wl * S::PW + p.lp;
+  p.on = p.lane < S::PW * N;
+  return p;
+}
+
+// line back to full precision in registers (per warp): the values of lines far below the slice's
+// largest entry gain the bits that the common exponent left unused
+template <int N>
+__device__ __forceinline__ void fix_widen(long long (&V)[N], int& E) {
+  unsigned m = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) m = fix_mag(m, V[i]);
+  const int sh = fix_renorm(m);
+  if (sh != 0) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) V[i] = fix_shift(V[i], sh);
+    E -= sh;
+  }
+}
+
+// One pass of a warp's lines: results to dst[i STEP], brought back into range there.
+template <int N, bool IN_SPEC, bool OUT_SPEC, int STEP>
+__device__ __forceinline__ void fix_pass(const long long (&V)[N], int& E, const LineCoefFix<N>& cf,
+                                         long long* dst, bool on) {
+  unsigned m = 0;
+  line_op_int<N, IN_SPEC, OUT_SPEC>(V, reinterpret_cast<const int4*>(cf.c),
+                                    [&](int i, long long val) {
+                                      m = fix_mag(m, val);
+                                      if (on) dst[i * STEP] = val;
+                                    });
+  const int sh = fix_renorm(m);
+  if (sh != 0) {
+    if (on)
+#pragma unroll 4
+      for (int i = 0; i < N; ++i) dst[i * STEP] = fix_shift(dst[i * STEP], sh);
+    E -= sh;
+  }
+}
+
+// The line operator along the three axes of a slice.  In: V, the line (line, lx) of the first
+// axis, exponent E of the warp.  With regions [line][i][lx] of padded rows:
+//   pass 0  first axis, results i to rows i of the warp's own regions;
+//   pass 1  x: lane (lp, lx) takes row lx of its region, in place;
+//   pass 2  the axis across the regions, for (row `line`, column lx): its input line in V, ready
+//           for line_op_int, exponent E (fix_two returns before it).
+template <int N, bool IN_SPEC, bool OUT_SPEC>
+__device__ __forceinline__ void fix_two(const FixPos<N>& p, bool on, long long (&V)[N], int& E,
+                                        const LineCoefFix<N> (&cf)[3], long long* sm, int* se_cta,
+                                        int rank) {
+  namespace cg = cooperative_groups;
+  using S = FixShape<N>;
+  long long* const mine = sm + p.line * S::PL;
+  fix_pass<N, IN_SPEC, OUT_SPEC, S::P>(V, E, cf[0], mine + p.lx, on);
+  __syncwarp();
+  long long* const row = mine + p.lx * S::P;
+#pragma unroll
+  for (int x = 0; x < N; ++x) V[x] = on ? row[x] : 0;
+  fix_pass<N, IN_SPEC, OUT_SPEC, 1>(V, E, cf[1], row, on);
+  int* const se_mine = se_cta + p.s * S::WPS;
+  if (p.lane == 0) se_mine[p.wl] = E;
+  int se[S::NTILE];
+  if constexpr (S::C > 1) {
+    cg::this_cluster().sync();
+    const int y = rank * S::NPC + p.line;
+#pragma unroll
+    for (int o = 0; o < S::C; ++o) {
+      const int* r = cg::this_cluster().map_shared_rank(se_cta, o);
+#pragma unroll
+      for (int w = 0; w < S::WPS; ++w) se[o * S::WPS + w] = r[w];
+    }
+    E = se[0];
+#pragma unroll
+    for (int i = 1; i < S::NTILE; ++i) E = max(E, se[i]);
+#pragma unroll
+    for (int o = 0; o < S::C; ++o) {
+      const long long* r = cg::this_cluster().map_shared_rank(sm, o) + y * S::P + p.lx;
+#pragma unroll
+      for (int k = 0; k < S::NPC; ++k)
+        V[o * S::NPC + k] = fix_align(r[k * S::PL], E - se[(o * S::NPC + k) / S::PW]);
+    }
+  } else {
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < S::NTILE; ++w) se[w] = se_mine[w];
+    E = se[0];
+#pragma unroll
+    for (int i = 1; i < S::NTILE; ++i) E = max(E, se[i]);
+    const long long* const col = sm + p.line * S::P + p.lx;
+#pragma unroll
+    for (int i = 0; i < N; ++i) V[i] = on ? fix_align(col[i * S::PL], E - se[i / S::PW]) : 0;
+  }
+  fix_widen<N>(V, E);
+}
+
+// Partial pair of the CTA and the fused scalar step (any number of threads up to 1024).
+__device__ __forceinline__ void fix_partials(double pd, double ps, double* partials, int fop,
+                                             const BatchTile* tiles, int unit,
+                                             const BatchProb* probs, DevScalars* scs,
+                                             unsigned* counters, int part_base) {
+  __shared__ double red[32][2];
+  const int tid = threadIdx.x, nw = (blockDim.x + 31) / 32;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    pd += __shfl_xor_sync(0xffffffffu, pd, o);
+    ps += __shfl_xor_sync(0xffffffffu, ps, o);
+  }
+  if ((tid & 31) == 0) {
+    red[tid >> 5][0] = pd;
+    red[tid >> 5][1] = ps;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    double d = 0.0, q = 0.0;
+    for (int w = 0; w < nw; ++w) {
+      d += red[w][0];
+      q += red[w][1];
+    }
+    partials[2 * blockIdx.x] = d;
+    partials[2 * blockIdx.x + 1] = q;
+  }
+  if (fop >= 0) {
+    if (tiles != nullptr) {
+      const int prob = tiles[unit].prob;
+      last_block_update_any(fop, scs + prob, partials, probs[prob].st0 - part_base,
+                            probs[prob].st1 - part_base, counters + prob);
+    } else {  // one lattice: the grid's last CTA
+      last_block_update_any(fop, scs, partials, 0, (int)gridDim.x, counters);
+    }
+  }
+}
+
+// Work unit of a CTA: its problem, time extent and this thread's output slice.
+struct FixUnit {
+  int t_out, ntau;
+  size_t off;
+  double acoef;
+  bool run, have;
+};
+template <int N, class Args>
+__device__ __forceinline__ FixUnit fix_unit(const Args& A, int unit, int s) {
+  FixUnit u;
+  int t0;
+  const int* done = A.done;
+  u.off = 0;
+  u.acoef = A.a;
+  if (A.tiles != nullptr) {
+    const BatchTile tl = A.tiles[unit];
+    const BatchProb& pr = A.probs[tl.prob];
+    t0 = tl.t0;
+    u.ntau = pr.ntau;
+    u.off = (size_t)pr.off;
+    done = pr.done;
+    if (A.scale_by_A) u.acoef *= pr.A;
+  } else {
+    t0 = unit * A.spc;
+    u.ntau = A.ntau;
+  }
+  u.run = !(done != nullptr && A.exec_if >= 0 && *done != A.exec_if);  // uniform per problem
+  u.t_out = t0 + s;
+  u.have = u.t_out < u.ntau;
+  return u;
+}
+
+template <int N>
+constexpr int fix_min_blocks() {
+  // N = 16 and 32: three CTAs (24 and 12 warps) per SM
+  return N == 32 ? 3 : N == 16 ? 3 : 1;
+}
+
+template <int N, int FAM, int EPI>
+__global__ void __launch_bounds__(FixShape<N>::NT, fix_min_blocks<N>())
+slice_fix_kernel(const __grid_constant__ FixArgs<N> A) {
+  pdl_begin();
+  namespace cg = cooperative_groups;
+  using S = FixShape<N>;
+  constexpr bool IN_SPEC = FAM == FAM_INV, OUT_SPEC = FAM == FAM_FWD;
+  constexpr int NN = N * N, VOL = N * NN, C = S::C;
+  extern __shared__ __align__(16) unsigned char fix_smem[];
+  __shared__ int se_all[S::MAXS * S::WPS];
+  __shared__ alignas(8) uint64_t bar2;
+  const FixPos<N> p = fix_pos<N>();
+  const int unit = blockIdx.x / C;
+  const FixUnit u = fix_unit<N>(A, unit, p.s);
+  if (!u.run) return;
+  int rank = 0;
+  if constexpr (C > 1) rank = (int)cg::this_cluster().block_rank();
+  if (A.expire && threadIdx.x == 0) mbar_expire_one_wait(&bar2, 256u, A.err);
+  const bool on = p.on && u.have;
+  long long* const sm = reinterpret_cast<long long*>(fix_smem) + (size_t)p.s * S::SLOT;
+  int t_in = u.t_out;
+  if (A.shift < 0) t_in = u.t_out == 0 ? u.ntau - 1 : u.t_out - 1;
+  if (A.shift > 0) t_in = u.t_out == u.ntau - 1 ? 0 : u.t_out + 1;
+  int E;
+  long long V[N];
+  {  // y-line (plane, x) from global memory
+    double v[N];
+    const int m0 = (rank * S::NPC + p.line) * NN + p.lx;  // site (or mode) of the line
+    const double* gi = A.in + u.off + (size_t)t_in * VOL + m0;
+#pragma unroll
+    for (int y = 0; y < N; ++y) v[y] = on ? __ldg(gi + y * N) : 0.0;
+    if (A.pre != nullptr) {
+      const double* gw = A.pre + u.off + (size_t)t_in * VOL + m0;
+#pragma unroll
+      for (int y = 0; y < N; ++y) v[y] *= on ? __ldg(gw + y * N) : 0.0;
+    }
+    if (A.bkpre != nullptr) {
+#pragma unroll
+      for (int y = 0; y < N; ++y) v[y] *= on ? __ldg(A.bkpre + m0 + y * N) : 0.0;
+    }
+    E = fix_tile<N>(v, V);
+  }
+  fix_two<N, IN_SPEC, OUT_SPEC>(p, on, V, E, A.cf, sm, se_all, rank);
+  double acc_dot = 0.0, acc_self = 0.0;
+  if (on) {  // last pass and epilogue: sites (z, y, x) of this thread's column
+    const FixOut fo = fix_out<N>(V, E, (A.shift < 0 && u.t_out != 0) ||
+                                           (A.shift > 0 && u.t_out != u.ntau - 1));
+    const double acoef = u.acoef;
+    const int q = (rank * S::NPC + p.line) * N + p.lx;
+    const size_t obase = u.off + (size_t)u.t_out * VOL + q;
+    auto site = [&](int z, double o) {
+      const size_t g = obase + (size_t)z * NN;
+      if constexpr (EPI == EPI_ANY || (EPI & E_UV) != 0) {  // U or V may alias out
+        if (A.bkpost != nullptr) o *= A.bkpost[z * NN + q];
+        if (A.post != nullptr) o *= A.post[g];
+        if (A.post2 != nullptr) o *= A.post2[g];
+        if (A.id != nullptr) o += A.id[g];
+        o *= acoef;
+        if (A.U != nullptr) o = fmadd(A.bU, A.U[g], o);
+        if (A.V != nullptr) o = fmadd(A.cV, A.V[g], o);
+      } else {  // unit scale (fix_launch_fam)
+        if constexpr ((EPI & E_BK) != 0) o *= __ldg(A.bkpost + z * NN + q);
+        if constexpr ((EPI & E_POST) != 0) o *= __ldg(A.post + g);
+        if constexpr ((EPI & E_ID) != 0) o += __ldg(A.id + g);
+      }
+      A.out[g] = o;
+      if constexpr ((EPI & E_DOT) != 0) {
+        if (A.want_dotP) acc_dot = fmadd(o, A.dotP[g], acc_dot);
+        if (A.want_self) acc_self = fmadd(o, o, acc_self);
+      }
+    };
+    line_op_int<N, IN_SPEC, OUT_SPEC>(
+        V, reinterpret_cast<const int4*>(A.cf[2].c),
+        [&](int z, long long iv) { site(z, fix_get(fo, iv)); });
+  }
+  if ((EPI & E_DOT) != 0 && (A.want_dotP || A.want_self))
+    fix_partials(acc_dot, acc_self, A.partials, A.fop, A.tiles, unit, A.probs, A.scs, A.counters,
+                 A.part_base);
+  if constexpr (C > 1) cg::this_cluster().sync();  // peers may still read this CTA's planes
+}
+
+// ---- the fused momentum-space kernels (FAM_M1W; see slice_m1w_kernel for the operators) ------
+// The inverse transform in the order y, x, z leaves each thread its z-column, which takes the site
+// multiplier and goes straight into the forward transform in the order z, x, y: the same three
+// exchanges again (fix_three), and the last pass ends with consecutive x for the epilogue.
+template <int N>
+struct FixM1wArgs {
+  LineCoefFix<N> ci[3], cf[3];  // inverse, forward transform, one copy per pass
+  const double* in;
+  const double* site;  // s or w
+  const double* bk;    // per-mode factor
+  double* out;
+  double a;
+  const int* done;
+  int exec_if;
+  const BatchTile* tiles;
+  const BatchProb* probs;
+  int scale_by_A;
+  int ntau, spc;
+  const double* U;
+  const double* dotP;
+  double full_scale, bU;
+  int want_dotP, want_self;
+  double* partials;
+  int fop;
+  DevScalars* scs;
+  unsigned* counters;
+  int part_base;
+  int* err;
+  int expire;
+};
+
+template <int N, int DIR, bool FULL>
+__global__ void __launch_bounds__(FixShape<N>::NT, fix_min_blocks<N>())
+slice_fix_m1w_kernel(const __grid_constant__ FixM1wArgs<N> A) {
+  pdl_begin();
+  using S = FixShape<N>;
+  static_assert(S::C == 1, "one CTA holds whole slices");
+  constexpr int NN = N * N, VOL = N * NN;
+  extern __shared__ __align__(16) unsigned char fix_smem[];
+  __shared__ int se_all[S::MAXS * S::WPS];
+  __shared__ alignas(8) uint64_t bar2;
+  const FixPos<N> p = fix_pos<N>();
+  const int unit = blockIdx.x;
+  const FixUnit u = fix_unit<N>(A, unit, p.s);
+  if (!u.run) return;
+  if (A.expire && threadIdx.x == 0) mbar_expire_one_wait(&bar2, 256u, A.err);
+  const bool on = p.on && u.have;
+  long long* const sm = reinterpret_cast<long long*>(fix_smem) + (size_t)p.s * S::SLOT;
+  const int t_in = DIR == 0 ? (u.t_out == 0 ? u.ntau - 1 : u.t_out - 1)
+                            : (u.t_out == u.ntau - 1 ? 0 : u.t_out + 1);
+  const bool neg = DIR == 0 ? u.t_out != 0 : u.t_out != u.ntau - 1;
+  const int t_s = DIR == 0 ? t_in : u.t_out;  // slice of the site multiplier
+  const int m0 = p.line * NN + p.lx;          // first mode of this thread's (plane, x) line
+  int E;
+  long long V[N];
+  {  // mode line (plane, x) from global memory
+    double v[N];
+    const double* gi = A.in + u.off + (size_t)t_in * VOL + m0;
+#pragma unroll
+    for (int y = 0; y < N; ++y) v[y] = on ? __ldg(gi + y * N) : 0.0;
+    if constexpr (DIR == 1) {
+#pragma unroll
+      for (int y = 0; y < N; ++y) v[y] *= on ? __ldg(A.bk + m0 + y * N) : 0.0;
+    }
+    E = fix_tile<N>(v, V);
+  }
+  fix_two<N, true, false>(p, on, V, E, A.ci, sm, se_all, 0);
+  {  // last inverse pass, site multiplier on the column (row `line`, x)
+    double v[N];
+    const FixOut fo = fix_out<N>(V, E, neg);
+    const double* gs = A.site + u.off + (size_t)t_s * VOL + p.line * N + p.lx;
+    line_op_int<N, true, false>(
+        V, reinterpret_cast<const int4*>(A.ci[2].c), [&](int z, long long iv) {
+          v[z] = on ? __ldg(gs + z * NN) * fix_get(fo, iv) : 0.0;
+        });
+    E = fix_tile<N>(v, V);
+  }
+  __syncthreads();  // every column has been read
+  fix_two<N, false, true>(p, on, V, E, A.cf, sm, se_all, 0);
+  double acc_dot = 0.0, acc_self = 0.0;
+  if (on) {  // last forward pass and epilogue: modes (plane, y, x)
+    const FixOut fo = fix_out<N>(V, E);
+    const double acoef = u.acoef, fs = A.full_scale;
+    const size_t so = u.off + (size_t)u.t_out * VOL;
+    auto mode = [&](int y, double o) {
+      const int g = m0 + y * N;
+      if constexpr (DIR == 0) o *= __ldg(A.bk + g);
+      if constexpr (FULL) {  // acoef = 1 (fix_m1w_launch)
+        o += __ldg(A.in + so + g);
+        if (A.U != nullptr) o = fmadd(fs, o, A.bU * A.U[so + g]);  // U may be out
+      } else {
+        o *= acoef;
+      }
+      A.out[so + g] = o;
+      if constexpr (FULL) {
+        if (A.want_dotP) acc_dot = fmadd(o, __ldg(A.dotP + so + g), acc_dot);
+        if (A.want_self) acc_self = fmadd(o, o, acc_self);
+      }
+    };
+    line_op_int<N, false, true>(V, reinterpret_cast<const int4*>(A.cf[2].c),
+                                [&](int y, long long iv) { mode(y, fix_get(fo, iv)); });
+  }
+  if constexpr (FULL) {
+    if (A.want_dotP || A.want_self)
+      fix_partials(acc_dot, acc_self, A.partials, A.fop, A.tiles, unit, A.probs, A.scs, A.counters,
+                   A.part_base);
+  }
+}
+
+// ---- launchers -------------------------------------------------------------------------------
+template <int N, class Args>
+inline void fix_common(Args& a, const SliceCall& c, cudaStream_t st) {
+  a.in = static_cast<const double*>(c.in);
+  a.out = static_cast<double*>(c.out);
+  a.U = static_cast<const double*>(c.U);
+  a.dotP = static_cast<const double*>(c.dotP);
+  a.a = c.a;
+  a.bU = c.bU;
+  a.partials = c.partials;
+  a.want_dotP = c.want_dotP;
+  a.want_self = c.want_self;
+  a.done = c.done;
+  a.exec_if = c.exec_if;
+  a.tiles = c.tiles;
+  a.probs = c.probs;
+  a.scale_by_A = c.scale_by_A;
+  a.ntau = c.ntau;
+  a.spc = c.spc < FixShape<N>::MAXS ? (c.spc < 1 ? 1 : c.spc) : FixShape<N>::MAXS;
+  a.fop = c.fop;
+  a.scs = c.scs;
+  a.counters = c.counters;
+  a.part_base = c.part_base;
+  a.err = c.err;
+  // the lattices whose FP32 or FP64 kernels stage by TMA carry the expiring wait
+  a.expire = (c.allow_tma && c.err != nullptr && (N == 8 || N == 16)) ? take_expired_wait(st) : 0;
+}
+
+// the launch of a kernel of this file: spc slices per CTA (cluster)
+template <int N, class Args>
+inline cudaError_t fix_launch(void (*kern)(Args), int* configured, const Args& a,
+                              const SliceCall& c, cudaStream_t st) {
+  using S = FixShape<N>;
+  if (c.tiles != nullptr && (c.spc > S::MAXS || S::C > 1)) return cudaErrorInvalidValue;
+  if ((c.want_dotP && c.dotP == nullptr) || ((c.want_dotP || c.want_self) && !c.partials) ||
+      (c.fop >= 0 && (c.scs == nullptr || c.counters == nullptr ||
+                      (c.tiles == nullptr && c.part_base != 0))))
+    return cudaErrorInvalidValue;
+  if (!*configured) {
+    cudaError_t e =
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(S::MAXS * S::SLOT * sizeof(long long)));
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+    *configured = 1;
+  }
+  const int units = c.tiles != nullptr ? c.ntiles : (c.ntau + a.spc - 1) / a.spc;
+  if (c.grid_out) *c.grid_out = units * S::C;
+  return launch_k(kern, dim3(units * S::C), dim3(a.spc * S::TS),
+                  (size_t)a.spc * S::SLOT * sizeof(long long), st, S::C, a);
+}
+
+template <int N, int FAM, int EPI>
+inline cudaError_t fix_launch_epi(const SliceCall& c, cudaStream_t st) {
+  FixArgs<N> a;
+  std::memset(&a, 0, sizeof(a));
+  for (int i = 0; i < 3; ++i) std::memcpy(&a.cf[i], c.coef, sizeof(a.cf[i]));
+  fix_common<N>(a, c, st);
+  a.pre = static_cast<const double*>(c.pre);
+  a.bkpre = static_cast<const double*>(c.bkpre);
+  a.bkpost = static_cast<const double*>(c.bkpost);
+  a.id = static_cast<const double*>(c.id);
+  a.post = static_cast<const double*>(c.post);
+  a.post2 = static_cast<const double*>(c.post2);
+  a.V = static_cast<const double*>(c.V);
+  a.cV = c.cV;
+  a.shift = c.shift;
+  static int configured = 0;
+  return fix_launch<N>(slice_fix_kernel<N, FAM, EPI>, &configured, a, c, st);
+}
+
+template <int N>
+inline cudaError_t fix_launch_fam(const SliceCall& c, cudaStream_t st) {
+  const int mask = (c.id ? E_ID : 0) | (c.post ? E_POST : 0) | (c.post2 ? E_POST2 : 0) |
+                   ((c.U || c.V) ? E_UV : 0) | ((c.want_dotP || c.want_self) ? E_DOT : 0) |
+                   (c.bkpost ? E_BK : 0);
+  // the variants without E_UV leave the scale out
+  if (c.a != 1.0 || c.scale_by_A) {
+    switch (c.fam) {
+      case FAM_KIN: return fix_launch_epi<N, FAM_KIN, EPI_ANY>(c, st);
+      case FAM_FWD: return fix_launch_epi<N, FAM_FWD, EPI_ANY>(c, st);
+    }
+    return fix_launch_epi<N, FAM_INV, EPI_ANY>(c, st);
+  }
+  if (c.fam == FAM_KIN) {
+    if (mask == E_ID) return fix_launch_epi<N, FAM_KIN, E_ID>(c, st);                      // M
+    if (mask == (E_ID | E_POST)) return fix_launch_epi<N, FAM_KIN, E_ID | E_POST>(c, st);  // M^T
+    if constexpr (N < 32) {
+      if (mask == (E_ID | E_DOT)) return fix_launch_epi<N, FAM_KIN, E_ID | E_DOT>(c, st);
+      if (mask == (E_ID | E_POST | E_DOT))
+        return fix_launch_epi<N, FAM_KIN, E_ID | E_POST | E_DOT>(c, st);
+    }
+    return fix_launch_epi<N, FAM_KIN, EPI_ANY>(c, st);
+  }
+  if (c.fam == FAM_FWD)
+    return mask == 0 ? fix_launch_epi<N, FAM_FWD, 0>(c, st)
+                     : fix_launch_epi<N, FAM_FWD, EPI_ANY>(c, st);
+  return mask == 0 ? fix_launch_epi<N, FAM_INV, 0>(c, st)
+                   : fix_launch_epi<N, FAM_INV, EPI_ANY>(c, st);
+}
+
+template <int N, int DIR, bool FULL>
+inline cudaError_t fix_m1w_launch(const SliceCall& c, cudaStream_t st) {
+  if (c.in == nullptr || c.pre == nullptr || c.out == nullptr || c.coef == nullptr ||
+      c.coef2 == nullptr || (DIR == 1 ? c.bkpre : c.bkpost) == nullptr ||
+      (FULL && (c.a != 1.0 || c.scale_by_A)))
+    return cudaErrorInvalidValue;
+  FixM1wArgs<N> a;
+  std::memset(&a, 0, sizeof(a));
+  for (int i = 0; i < 3; ++i) {
+    std::memcpy(&a.ci[i], c.coef, sizeof(a.ci[i]));
+    std::memcpy(&a.cf[i], c.coef2, sizeof(a.cf[i]));
+  }
+  fix_common<N>(a, c, st);
+  a.site = static_cast<const double*>(c.pre);
+  a.bk = static_cast<const double*>(DIR == 1 ? c.bkpre : c.bkpost);
+  a.full_scale = c.full_scale;
+  static int configured = 0;
+  return fix_launch<N>(slice_fix_m1w_kernel<N, DIR, FULL>, &configured, a, c, st);
+}
+
+// FP64 slice launch of a 3-D lattice.
+template <int N>
+inline cudaError_t slice_fix_try(const SliceCall& c, cudaStream_t st) {
+  if (c.fam != FAM_M1W) return fix_launch_fam<N>(c, st);
+  if constexpr (FixShape<N>::C == 1) {
+    if (c.shift < 0)
+      return c.m1w_full ? fix_m1w_launch<N, 0, true>(c, st) : fix_m1w_launch<N, 0, false>(c, st);
+    return c.m1w_full ? fix_m1w_launch<N, 1, true>(c, st) : fix_m1w_launch<N, 1, false>(c, st);
+  }
+  return cudaErrorNotSupported;
+}
+
+}  // namespace ufg

@@ -2,7 +2,7 @@
 // supported N so the heavy unrolled kernels build in parallel).
 #include <cstdlib>
 
-#include "slice_df.cuh"
+#include "slice_fix.cuh"
 #include "slice_kernel.cuh"
 #include "slice_pair.cuh"
 #include "slice_lowd.cuh"
@@ -28,6 +28,8 @@ static bool tma_enabled() {
 template <>
 cudaError_t slice_launch<UFG_N>(const SliceCall& c, cudaStream_t st) {
   if (c.dim != 3) return slice_lowd_try<UFG_N>(c, st);       // 1-D and 2-D lattices
+  if (c.prec == 0)  // the integer-pipe kernels, but for the 32^3 calls that keep the FP64 pipe
+    return c.fp64_pipe ? slice_launch_fp64<UFG_N>(c, st) : slice_fix_try<UFG_N>(c, st);
   if (c.fam == FAM_M1W) return slice_m1w_try<UFG_N>(c, st);  // callers check support first
   if (c.fam == FAM_Q) return slice_q_try<UFG_N>(c, st);      // callers check support first
   if (c.allow_tma && tma_enabled()) {
@@ -41,7 +43,7 @@ cudaError_t slice_launch<UFG_N>(const SliceCall& c, cudaStream_t st) {
 template <>
 bool slice_tma_prep_ok<UFG_N>(int prec, int allow_tma) {
   if (!allow_tma || !tma_enabled()) return false;
-  return prec == 1 ? (UFG_N == 16 || UFG_N == 32) : (UFG_N == 8 || UFG_N == 16);
+  return prec == 1 && (UFG_N == 16 || UFG_N == 32);
 }
 
 }  // namespace ufg

@@ -1,4 +1,5 @@
-// The fused per-time-slice kernel behind every apply of the fermion matrix family.
+// The fused per-time-slice kernel behind the FP32 applies of the fermion matrix family on lattices
+// without a TMA shape (FP64: slice_fix.cuh).
 //
 // One CTA (or one thread-block cluster of C CTAs for the largest slices) owns `spc` consecutive
 // output time slices.  For each it
@@ -105,7 +106,7 @@ constexpr int E_IDB = 256;
 // Resident CTAs per SM the register allocation must allow (256 threads each).
 template <int N, typename R>
 constexpr int slice_min_blocks() {
-  return N >= 32 ? (sizeof(R) == 4 ? 3 : 1) : (N >= 16 ? (sizeof(R) == 4 ? 3 : 2) : 3);
+  return N >= 32 && sizeof(R) == 8 ? 1 : 3;
 }
 
 template <int N, typename R, int C, int FAM, int EPI>
@@ -424,27 +425,26 @@ inline cudaError_t launch_C(const SliceCall& c, cudaStream_t st) {
     if (c.C == 4) return launch_one<N, R, 4, FAM>(c, st);
     if (c.C == 2) return launch_one<N, R, 2, FAM>(c, st);
   }
-  if (c.C == 1) {
-    // an FP64 32^3 slice (270 KB padded) exceeds one CTA's shared memory
-    if constexpr (N < 32 || sizeof(R) == 4) return launch_one<N, R, 1, FAM>(c, st);
-  }
+  if (c.C == 1) return launch_one<N, R, 1, FAM>(c, st);
   return cudaErrorInvalidValue;
+}
+
+// The FP64-pipe form, for the 32^3 calls whose results are to keep their bits (SliceCall::
+// fp64_pipe): the kinetic family in clusters of four CTAs.
+template <int N>
+cudaError_t slice_launch_fp64(const SliceCall& c, cudaStream_t st) {
+  if constexpr (N == 32) {
+    if (c.fam == FAM_KIN && c.tiles == nullptr) return launch_one<N, double, 4, FAM_KIN>(c, st);
+  }
+  return cudaErrorNotSupported;
 }
 
 template <int N>
 cudaError_t slice_launch_plain(const SliceCall& c, cudaStream_t st) {
-  if (c.prec == 0) {
-    switch (c.fam) {
-      case FAM_KIN: return launch_C<N, double, FAM_KIN>(c, st);
-      case FAM_FWD: return launch_C<N, double, FAM_FWD>(c, st);
-      case FAM_INV: return launch_C<N, double, FAM_INV>(c, st);
-    }
-  } else {
-    switch (c.fam) {
-      case FAM_KIN: return launch_C<N, float, FAM_KIN>(c, st);
-      case FAM_FWD: return launch_C<N, float, FAM_FWD>(c, st);
-      case FAM_INV: return launch_C<N, float, FAM_INV>(c, st);
-    }
+  switch (c.fam) {
+    case FAM_KIN: return launch_C<N, float, FAM_KIN>(c, st);
+    case FAM_FWD: return launch_C<N, float, FAM_FWD>(c, st);
+    case FAM_INV: return launch_C<N, float, FAM_INV>(c, st);
   }
   return cudaErrorInvalidValue;
 }

@@ -13,7 +13,7 @@
 // launch instead of two and no intermediate vector in memory: at 16^3 the two launches are
 // bound by latency (one CTA per slice, few CTAs per SM), not by their bytes.  The multiplier
 // rows of the x-passes come from global memory (16-byte loads), the epilogue's w_t per site.
-// Built for 16^3 slices (FP32 and FP64); slice_q_supported says where it runs.
+// Built for FP32 16^3 slices; slice_q_supported says where it runs.
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -46,8 +46,7 @@ struct QArgs {
 
 template <int N, typename R>
 constexpr int q_min_blocks() {
-  // three boxes of one slice: FP32 16^3 48 KB (four CTAs per SM), FP64 16^3 96 KB (two)
-  return (3 * N * N * N * (int)sizeof(R) + 1024) <= 56 * 1024 ? 4 : 2;
+  return 4;  // three boxes of one 16^3 slice: 48 KB
 }
 
 // x-pass in place: rows of X (times the multiplier rows of wg when given)
@@ -251,11 +250,11 @@ inline cudaError_t q_launch_epi(const SliceCall& c, cudaStream_t st) {
   return dot ? q_launch<N, R, false, true>(c, st) : q_launch<N, R, false, false>(c, st);
 }
 
-// The fused Q for 16^3 slices (FP32 and FP64), where the one-CTA TMA boxes hold one slice.
+// The fused Q for FP32 16^3 slices, where the one-CTA TMA boxes hold one slice.
 template <int N>
 cudaError_t slice_q_try(const SliceCall& c, cudaStream_t st) {
   if constexpr (N == 16) {
-    return c.prec == 1 ? q_launch_epi<16, float>(c, st) : q_launch_epi<16, double>(c, st);
+    if (c.prec == 1) return q_launch_epi<16, float>(c, st);
   }
   return cudaErrorNotSupported;
 }

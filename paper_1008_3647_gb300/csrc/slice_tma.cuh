@@ -1,5 +1,5 @@
 // TMA-staged form of the slice kernel for the shapes whose rows are one 64- or 128-byte swizzle
-// span (FP32 N = 16, 32; FP64 N = 8, 16).
+// span (FP32 N = 16, 32).
 //
 // Each CTA (or cluster of C CTAs splitting a slice's z-planes) handles one work unit (a time
 // slice, or a (problem, slice) tile of a batch).  Its planes -- and those of the per-site load
@@ -138,10 +138,6 @@ __device__ __forceinline__ void mul_chunk(float (&v)[4], const float (&w)[4]) {
   v[2] = b.x;
   v[3] = b.y;
 }
-__device__ __forceinline__ void mul_chunk(double (&v)[2], const double (&w)[2]) {
-  v[0] *= w[0];
-  v[1] *= w[1];
-}
 
 // A store into another CTA's shared memory through its 32-bit shared::cluster address (mapa).
 __device__ __forceinline__ uint32_t cluster_addr(const void* p, int rank) {
@@ -151,9 +147,6 @@ __device__ __forceinline__ uint32_t cluster_addr(const void* p, int rank) {
 }
 __device__ __forceinline__ void st_cluster(uint32_t a, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v));
-}
-__device__ __forceinline__ void st_cluster(uint32_t a, double v) {
-  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v));
 }
 
 // x-pass output: the row's N results are collected in registers and written back as 16-byte
@@ -196,7 +189,7 @@ constexpr uint32_t EXPIRE_LIMIT = 1u << 8;     // rounds of the wait ufg_test_ex
 // Resident CTAs per SM the register allocation must allow.
 template <int N, typename R>
 constexpr int tma_min_blocks() {
-  return sizeof(R) == 4 ? (N == 16 ? 5 : 3) : (N <= 8 ? 4 : 3);
+  return N == 16 ? 5 : 3;
 }
 
 // Threads per CTA: 256, except for 8-CTA clusters of 32^3 slices (four z-planes per CTA, one
@@ -767,7 +760,7 @@ struct M1wArgs {
 
 template <int N, typename R>
 constexpr int m1w_min_blocks() {
-  return sizeof(R) == 4 ? 5 : (N <= 8 ? 4 : 2);  // DIR 1 (three boxes) fits 4 by shared memory
+  return 5;  // DIR 1 (three boxes) fits 4 by shared memory
 }
 
 // Row-pair permutation of the one-CTA boxes with 64-byte rows and 16 rows per plane (FP32
@@ -1070,19 +1063,10 @@ inline cudaError_t m1w_dir(const SliceCall& c, cudaStream_t st) {
 }
 
 template <int N>
-cudaError_t m1w_df_try(const SliceCall& c, cudaStream_t st);
-
-template <int N>
 inline cudaError_t slice_m1w_try(const SliceCall& c, cudaStream_t st) {
   if (!slice_m1w_supported(N, c.prec) || c.shift == 0) return cudaErrorNotSupported;
-  if (c.emulate64 && c.prec == 0) return m1w_df_try<N>(c, st);
-  if constexpr (N == 16) {
-    if (c.prec == 1) return c.m1w_full ? m1w_dir<16, float, true>(c, st)
-                                       : m1w_dir<16, float, false>(c, st);
-    return c.m1w_full ? m1w_dir<16, double, true>(c, st) : m1w_dir<16, double, false>(c, st);
-  } else if constexpr (N == 8) {
-    return c.m1w_full ? m1w_dir<8, double, true>(c, st) : m1w_dir<8, double, false>(c, st);
-  }
+  if constexpr (N == 16)
+    return c.m1w_full ? m1w_dir<16, float, true>(c, st) : m1w_dir<16, float, false>(c, st);
   return cudaErrorNotSupported;
 }
 
@@ -1125,14 +1109,6 @@ inline cudaError_t slice_tma_try(const SliceCall& c, cudaStream_t st) {
         case FAM_KIN: return tma_launch_fam<N, float, C, FAM_KIN>(c, st);
         case FAM_FWD: return tma_launch_fam<N, float, C, FAM_FWD>(c, st);
         case FAM_INV: return tma_launch_fam<N, float, C, FAM_INV>(c, st);
-      }
-    }
-  } else {
-    if constexpr (N == 8 || N == 16) {
-      switch (c.fam) {
-        case FAM_KIN: return tma_launch_fam<N, double, 1, FAM_KIN>(c, st);
-        case FAM_FWD: return tma_launch_fam<N, double, 1, FAM_FWD>(c, st);
-        case FAM_INV: return tma_launch_fam<N, double, 1, FAM_INV>(c, st);
       }
     }
   }

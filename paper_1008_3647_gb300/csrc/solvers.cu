@@ -45,6 +45,7 @@ struct ufg_solver {
   int pc_kind = UFG_PC_NONE;
   ufg_pc_params pc = {};
   VecSet vs[2];
+  bool fp64_pipe = false;   // inside a mixed solve (kin_call)
   double* x64 = nullptr;    // FP64 solution accumulator (outer loops, host staging)
   double* b64 = nullptr;    // FP64 right-hand side staging
   double* r64 = nullptr;    // FP64 residual (outer loops, true residual)
@@ -112,6 +113,12 @@ LaunchWork vec_work(const ufg_solver* S, int prec, int op, long long n, const vo
 }
 
 double* slot(ufg_solver* S, int k) { return S->parts + (size_t)k * 2 * MAX_PARTIAL_CTAS; }
+
+// The kinetic family in precision prec; the FP64 calls of a mixed solve keep their bits on 32^3
+// lattices (base_call_fp64).
+SliceCall kin_call(const ufg_solver* S, const ufg_lattice* L, int prec) {
+  return prec == 0 && S->fp64_pipe ? base_call_fp64(L) : base_call(L, FAM_KIN, prec);
+}
 
 // ---- operator applications with epilogues --------------------------------------------------
 // out = a * (A in) + bU * U   with partials (out . dotP, out . out) into `part` when requested.
@@ -194,7 +201,7 @@ ufg_status apply_op(ufg_solver* S, const ufg_field* f, int prec, int op, const v
   }
   if (op == OPK_Q) {
     void* t1 = S->vs[prec].tmp;
-    SliceCall c = base_call(L, FAM_KIN, prec);
+    SliceCall c = kin_call(S, L, prec);
     c.in = in;
     c.pre = fld(f, 'w', prec);
     c.id = in;
@@ -207,7 +214,7 @@ ufg_status apply_op(ufg_solver* S, const ufg_field* f, int prec, int op, const v
     op = OPK_MDAG;
     S->counts.M++;
   }
-  SliceCall c = base_call(L, FAM_KIN, prec);
+  SliceCall c = kin_call(S, L, prec);
   c.in = in;
   c.id = in;
   if (op == OPK_M) {
@@ -712,9 +719,10 @@ ufg_status write_scalars(ufg_solver* S, double tol, int maxit, double div_limit 
 std::string key_of(const char* kind, ufg_solver* S, const ufg_field* f, int prec, int op,
                    int reps) {
   char buf[256];
-  snprintf(buf, sizeof(buf), "%s|%llu|%d|%d|%d|%d|%d|%g|%g|%g|%d|%d|%.17g|%.17g|%d", kind, f->id,
+  snprintf(buf, sizeof(buf), "%s|%llu|%d|%d|%d|%d|%d|%g|%g|%g|%d|%d|%.17g|%.17g|%d|%d", kind, f->id,
            prec, op, reps, S->pc_kind, S->pc.degree, S->pc.eps, S->pc.scale, S->pc.alpha,
-           S->pc.order, S->pc.euler, S->pc.euler_p, S->pc.vw_s, S->mom ? 1 : 0);
+           S->pc.order, S->pc.euler, S->pc.euler_p, S->pc.vw_s, S->mom ? 1 : 0,
+           S->fp64_pipe ? 1 : 0);
   return buf;
 }
 
@@ -1085,6 +1093,11 @@ bool momentum_basis(const ufg_solver* S, const ufg_field* f, int op, const ufg_p
 // solve, x = F^T x^.
 ufg_status solve_system(ufg_solver* S, ufg_field* f, int op, const double* rhs, double* x64,
                         bool x0, double tol, const ufg_params* p, SolveOut* out) {
+  struct Pipe {  // the FP64 residuals of a mixed solve (kin_call)
+    ufg_solver* S;
+    Pipe(ufg_solver* s, bool on) : S(s) { S->fp64_pipe = on; }
+    ~Pipe() { S->fp64_pipe = false; }
+  } pipe(S, p->precision == UFG_MIXED);
   if (!momentum_basis(S, f, op, p)) return solve_in_basis(S, f, op, rhs, x64, x0, tol, p, out);
   UFG_TRY(fourier64(S, f, rhs, S->mb64, false));
   if (x0) UFG_TRY(fourier64(S, f, x64, S->mx64, false));
@@ -1494,6 +1507,12 @@ ufg_status ufg_solve_bicgstab_two_step(ufg_solver* S, ufg_field* f, const double
     // one defect-correction round on the composite residual: x += two_step(b - Q x)
     ++extra;
     const size_t bytes = (size_t)S->lat->S * sizeof(double);
+    if (p->precision == UFG_MIXED && S->lat->nx == 32) {  // its right-hand side, see kin_call
+      S->fp64_pipe = true;
+      const ufg_status rs = residual64(S, f, OPK_Q, xd, bd, S->r64, &rn);
+      S->fp64_pipe = false;
+      UFG_TRY(rs);
+    }
     UFG_CUDA(cudaMemcpyAsync(S->rc64, S->r64, bytes, cudaMemcpyDeviceToDevice, S->st));
     UFG_CUDA(cudaMemcpyAsync(S->xs64, xd, bytes, cudaMemcpyDeviceToDevice, S->st));
     SolveOut c1, c2;
@@ -1680,7 +1699,7 @@ ufg_status ufg_hmc_trajectory(ufg_solver* S, ufg_field* f, const double* eta, co
     UFG_CUDA(cudaMemcpyAsync(sig, f->sigma, n * sizeof(double), cudaMemcpyDeviceToDevice, S->st));
     UFG_CUDA(cudaMemcpyAsync(pi, pi0, n * sizeof(double), cudaMemcpyDefault, S->st));
     // heat bath of the pseudofermions: phi = M^T eta, so that S_p = |eta|^2 at the start
-    UFG_TRY(op_Mdag(f, 0, eta, phi, S->st));
+    UFG_TRY(op_Mdag(f, 0, eta, phi, S->st, true));
     UFG_TRY(norm64(S, pi, n, &hs.H_old));
     hs.H_old = 0.5 * hs.H_old * hs.H_old;
   }

@@ -153,6 +153,7 @@ struct ufg_lattice {
   long long V = 0, S = 0;
   std::vector<double> lam;                 // exp(-tau E1) per 1-D spectral slot
   std::vector<unsigned char> coef[3][2];   // reduced line matrices [family][0 FP64 / 1 FP32]
+  std::vector<unsigned char> coef_fix[3];  // the FP64 matrices in fixed point (fix_ops.cuh)
   double* bk64 = nullptr;                  // per-mode exp(-tau E(k)), spectral layout [V]
   float* bk32 = nullptr;
   int* dev_err = nullptr;                  // device flag of bounded waits that ran out
@@ -189,9 +190,12 @@ namespace ufg {
 
 // Generic slice-kernel call prefilled for a field/lattice and precision.
 SliceCall base_call(const ufg_lattice* lat, int fam, int prec);
+// The FP64 kinetic family with the line passes of 32^3 lattices on the FP64 pipe (lattice.cu).
+SliceCall base_call_fp64(const ufg_lattice* lat);
 // Operator applications used by the C ABI and by the solvers (vectors in precision prec).
 ufg_status op_M(const ufg_field* f, int prec, const void* x, void* y, cudaStream_t st);
-ufg_status op_Mdag(const ufg_field* f, int prec, const void* x, void* y, cudaStream_t st);
+ufg_status op_Mdag(const ufg_field* f, int prec, const void* x, void* y, cudaStream_t st,
+                   bool fp64_pipe = false);
 ufg_status op_M0inv(const ufg_field* f, int prec, const void* x, void* y, void* tmp, int transpose,
                     cudaStream_t st);
 ufg_status ensure_sca(ufg_field* f, double alpha, cudaStream_t st);

@@ -362,7 +362,7 @@ def ufg_fourier(field, x, inverse=False, y=None):
 
 def ufg_apply_M_momentum(field, x, transpose=False, y=None, emulated=False):
     """M (or M^T) in the momentum basis: F M F^T x per slice-stacked vector.  emulated=True (FP64
-    vectors only): double-float arithmetic on the FP32 pipe."""
+    vectors only): UFG_FP64_EMULATED, the same kernel."""
     if not emulated:
         return _apply_flag("ufg_apply_M_momentum", field, x, transpose, y)
     _vec(x, field.lattice.shape, (torch.float64,))
