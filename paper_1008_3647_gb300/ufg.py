@@ -223,19 +223,28 @@ def _check(status):
         raise UfgError(status, load().ufg_last_error().decode())
 
 
-def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+# The raw handle of the current device's current stream.  torch.cuda.current_stream() builds a
+# Stream object around it (2.9 us a call, more than the whole C call of a small apply).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", None)
+if _raw_stream is None or _device is None:
+    def _stream():
+        return torch.cuda.current_stream().cuda_stream
+else:
+    def _stream():
+        return _raw_stream(_device())
 
 
+# Pointers and streams are passed as plain integers: the argument types of _SIGS convert them.
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
 
 
 def _vec(t, shape, dtypes=(torch.float64, torch.float32), host_ok=False):
     if not isinstance(t, torch.Tensor) or not t.is_contiguous() or not (t.is_cuda or host_ok):
         raise ValueError("vectors must be contiguous CUDA tensors" +
                          (" (or host tensors)" if host_ok else ""))
-    if tuple(t.shape) != tuple(shape) or t.dtype not in dtypes:
+    if t.shape != shape or t.dtype not in dtypes:
         raise ValueError("expected shape %s dtype in %s, got %s %s" % (shape, dtypes, tuple(t.shape),
                                                                        t.dtype))
     return t
@@ -255,11 +264,12 @@ class Lattice:
         self._h = h
         self.nx, self.ntau, self.tau, self.g, self.dispersion = nx, ntau, tau, g, dispersion
         self.dim = dim
+        self._shape = (ntau,) + (nx,) * dim
         self.A = lib.ufg_lattice_coupling(h)
 
     @property
     def shape(self):
-        return (self.ntau,) + (self.nx,) * self.dim
+        return self._shape
 
     def ufg_lattice_autotune(self):
         _check(load().ufg_lattice_autotune(self._h, _stream()))
@@ -303,13 +313,29 @@ class Field:
             self._h = None
 
 
-def _apply(name, field, x, y=None):
-    _vec(x, field.lattice.shape)
+_PREC = {torch.float64: UFG_FP64, torch.float32: UFG_FP32}
+
+
+def _operands(field, x, y):
+    """(y, precision, pointers) of an apply: x and y contiguous CUDA vectors of the lattice, one
+    dtype.  The common case is tested in line; _vec names what is wrong with the others."""
+    shape = field.lattice._shape
+    dtype = x.dtype if isinstance(x, torch.Tensor) else None
+    if dtype not in _PREC or x.shape != shape or not x.is_cuda or not x.is_contiguous():
+        _vec(x, shape)
     if y is None:
         y = torch.empty_like(x)
-    _vec(y, field.lattice.shape, (x.dtype,))
-    prec = UFG_FP64 if x.dtype == torch.float64 else UFG_FP32
-    _check(getattr(load(), name)(field._h, _ptr(x), _ptr(y), prec, _stream()))
+    elif (not isinstance(y, torch.Tensor) or y.dtype is not dtype or y.shape != shape or
+          not y.is_cuda or not y.is_contiguous()):
+        _vec(y, shape, (dtype,))
+    return y, _PREC[dtype], x.data_ptr(), y.data_ptr()
+
+
+def _apply(name, field, x, y=None):
+    y, prec, xp, yp = _operands(field, x, y)
+    status = getattr(_lib or load(), name)(field._h, xp, yp, prec, _stream())
+    if status != UFG_OK:
+        _check(status)
     return y
 
 
@@ -346,12 +372,10 @@ def ufg_apply_M0invT(field, x, y=None):
 
 
 def _apply_flag(name, field, x, flag, y=None):
-    _vec(x, field.lattice.shape)
-    if y is None:
-        y = torch.empty_like(x)
-    _vec(y, field.lattice.shape, (x.dtype,))
-    prec = UFG_FP64 if x.dtype == torch.float64 else UFG_FP32
-    _check(getattr(load(), name)(field._h, _ptr(x), _ptr(y), prec, int(flag), _stream()))
+    y, prec, xp, yp = _operands(field, x, y)
+    status = getattr(_lib or load(), name)(field._h, xp, yp, prec, int(flag), _stream())
+    if status != UFG_OK:
+        _check(status)
     return y
 
 
