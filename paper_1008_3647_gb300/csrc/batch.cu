@@ -86,6 +86,12 @@ struct Batch {
   double* parts = nullptr;
   size_t part_stride = 0;
   cudaStream_t st = nullptr;
+  // The groups' chains of slice and recurrence kernels touch disjoint problems, so they run side
+  // by side between two launches of the whole batch (for_groups): gs is the stream of the group
+  // being launched, fork_st the streams of the groups after the first.
+  cudaStream_t gs = nullptr;
+  std::vector<cudaStream_t> fork_st;
+  std::vector<cudaEvent_t> fork_ev;  // [0] fork, [i] join of fork_st[i - 1]
   int pc_kind = UFG_PC_NONE;
   ufg_pc_params pc = {};
   std::map<std::string, cudaGraphExec_t> graphs;
@@ -100,6 +106,8 @@ struct Batch {
     if (scs_h) cudaFreeHost(scs_h);
     if (scale_h) cudaFreeHost(scale_h);
     for (auto& g : groups) ufg_lattice_destroy(g.lat);
+    for (cudaEvent_t e : fork_ev) cudaEventDestroy(e);
+    for (cudaStream_t f : fork_st) cudaStreamDestroy(f);
     if (st) cudaStreamDestroy(st);
   }
   template <typename T>
@@ -136,6 +144,36 @@ LaunchWork batch_work(Batch& B, const std::vector<int>* idx, int exec_if, double
   return w;
 }
 
+// f(g) for every group, each on a stream of its own between the work before and after on B.st
+// (event fork and join; inside a capture these become parallel branches of the graph).  One
+// problem size fills the GPU poorly: the 96-problem batch has four groups whose kernels of 100
+// to 400 CTAs took 12 to 20 us one after the other.  In instrumented runs one after the other on
+// B.st, so that the kernels are timed alone.
+ufg_status for_groups(Batch& B, const std::function<ufg_status(Group&)>& f) {
+  const size_t n = B.groups.size();
+  B.gs = B.st;
+  if (n == 1 || profiling()) {
+    for (auto& g : B.groups) UFG_TRY(f(g));
+    return UFG_OK;
+  }
+  const size_t nf = B.fork_st.size();  // made by setup, before any capture
+  UFG_CUDA(cudaEventRecord(B.fork_ev[0], B.st));
+  for (size_t i = 0; i < nf; ++i) UFG_CUDA(cudaStreamWaitEvent(B.fork_st[i], B.fork_ev[0], 0));
+  ufg_status s = UFG_OK;
+  for (size_t i = 0; i < n && s == UFG_OK; ++i) {
+    const size_t k = i % (nf + 1);
+    B.gs = k == 0 ? B.st : B.fork_st[k - 1];
+    s = f(B.groups[i]);
+  }
+  B.gs = B.st;
+  for (size_t i = 0; i < nf; ++i) {  // joined also after a failure: a capture must end whole
+    UFG_CUDA(cudaEventRecord(B.fork_ev[i + 1], B.fork_st[i]));
+    UFG_CUDA(cudaStreamWaitEvent(B.st, B.fork_ev[i + 1], 0));
+  }
+  return s;
+}
+
+// on B.gs
 ufg_status slice(Batch& B, Group& g, SliceCall c, int exec_if) {
   c.tiles = g.tiles;
   c.ntiles = g.ntiles;
@@ -149,58 +187,33 @@ ufg_status slice(Batch& B, Group& g, SliceCall c, int exec_if) {
     c.part_base = g.cta_base;
   }
   note_launches(1);
-  KTimer kt(slice_kernel_name(c, g.lat->nx), B.st,
+  KTimer kt(slice_kernel_name(c, g.lat->nx), B.gs,
             batch_work(B, &g.probs, exec_if, slice_bytes_per_site(c),
                        slice_bytes_per_problem(c, g.lat->nx)));
-  cudaError_t e = slice_dispatch(g.lat->nx, c, B.st);
+  cudaError_t e = slice_dispatch(g.lat->nx, c, B.gs);
   if (e != cudaSuccess) return cuda_fail(e, "batched slice kernel");
   return UFG_OK;
 }
 
-// out = a * (A in) + bU * U with partials (out.dotP, out.out), all groups; fop >= 0 applies that
+// out = a * (A in) + bU * U with partials (out.dotP, out.out), one group or all; fop >= 0 applies that
 // scalar op to each problem from the partials in the same launch
-ufg_status apply_b(Batch& B, int prec, int op, const void* in, void* out, double a, const void* U,
-                   double bU, const void* dotP, bool self, double* part, int exec_if,
-                   int fop = -1) {
-  if (B.mom) {  // the fused momentum-space operator, one kernel per group
-    for (auto& g : B.groups) {
-      SliceCall c = base_call(g.lat, FAM_INV, prec);
-      c.fam = FAM_M1W;
-      c.coef2 = base_call(g.lat, FAM_FWD, prec).coef;
-      c.m1w_full = 1;
-      c.in = in;
-      c.pre = fldb(B, 'w', prec);
-      const void* bk = prec ? (const void*)g.lat->bk32 : (const void*)g.lat->bk64;
-      if (op == BOP_M) c.bkpost = bk;
-      else c.bkpre = bk;
-      c.shift = op == BOP_M ? -1 : +1;
-      c.a = 1.0;
-      c.full_scale = a;
-      c.out = out;
-      c.U = U;
-      c.bU = bU;
-      c.dotP = dotP;
-      c.want_dotP = dotP != nullptr;
-      c.want_self = self;
-      c.partials = part;
-      c.fop = fop;
-      UFG_TRY(slice(B, g, c, exec_if));
-    }
-    return UFG_OK;
-  }
-  for (auto& g : B.groups) {
-    SliceCall c = base_call(g.lat, FAM_KIN, prec);
+ufg_status apply_g(Batch& B, Group& g, int prec, int op, const void* in, void* out, double a,
+                   const void* U, double bU, const void* dotP, bool self, double* part,
+                   int exec_if, int fop) {
+  if (B.mom) {  // the fused momentum-space operator
+    SliceCall c = base_call(g.lat, FAM_INV, prec);
+    c.fam = FAM_M1W;
+    c.coef2 = base_call(g.lat, FAM_FWD, prec).coef;
+    c.m1w_full = 1;
     c.in = in;
-    c.id = in;
-    if (op == BOP_M) {
-      c.pre = fldb(B, 'w', prec);
-      c.shift = -1;
-    } else {
-      c.post = fldb(B, 'w', prec);
-      c.shift = +1;
-    }
+    c.pre = fldb(B, 'w', prec);
+    const void* bk = prec ? (const void*)g.lat->bk32 : (const void*)g.lat->bk64;
+    if (op == BOP_M) c.bkpost = bk;
+    else c.bkpre = bk;
+    c.shift = op == BOP_M ? -1 : +1;
+    c.a = 1.0;
+    c.full_scale = a;
     c.out = out;
-    c.a = a;
     c.U = U;
     c.bU = bU;
     c.dotP = dotP;
@@ -208,9 +221,35 @@ ufg_status apply_b(Batch& B, int prec, int op, const void* in, void* out, double
     c.want_self = self;
     c.partials = part;
     c.fop = fop;
-    UFG_TRY(slice(B, g, c, exec_if));
+    return slice(B, g, c, exec_if);
   }
-  return UFG_OK;
+  SliceCall c = base_call(g.lat, FAM_KIN, prec);
+  c.in = in;
+  c.id = in;
+  if (op == BOP_M) {
+    c.pre = fldb(B, 'w', prec);
+    c.shift = -1;
+  } else {
+    c.post = fldb(B, 'w', prec);
+    c.shift = +1;
+  }
+  c.out = out;
+  c.a = a;
+  c.U = U;
+  c.bU = bU;
+  c.dotP = dotP;
+  c.want_dotP = dotP != nullptr;
+  c.want_self = self;
+  c.partials = part;
+  c.fop = fop;
+  return slice(B, g, c, exec_if);
+}
+ufg_status apply_b(Batch& B, int prec, int op, const void* in, void* out, double a, const void* U,
+                   double bU, const void* dotP, bool self, double* part, int exec_if,
+                   int fop = -1) {
+  return for_groups(B, [&](Group& g) {
+    return apply_g(B, g, prec, op, in, out, a, U, bU, dotP, self, part, exec_if, fop);
+  });
 }
 
 ufg_status vecb(Batch& B, int prec, int op, int exec_if, const void* a, const void* b,
@@ -237,10 +276,10 @@ ufg_status scalb(Batch& B, int op, const double* part, int kind, const double* p
   return UFG_OK;
 }
 
-// z = P_d r (tr: P_d^T) for every running problem, momentum-space evaluation (see solvers.cu).
+// z = P_d r (tr: P_d^T) for every running problem of a group, momentum-space evaluation (see solvers.cu).
 // prep_r != nullptr: r is BiCGStab's direction p, first updated in place to
 // p = prep_r + beta (p - omega prep_v) by the forward transform (slice_tma_prep_supported).
-ufg_status wce_b(Batch& B, int prec, const void* r, void* z, bool tr,
+ufg_status wce_g(Batch& B, Group& g, int prec, const void* r, void* z, bool tr,
                  const void* prep_r = nullptr, const void* prep_v = nullptr) {
   const int d = B.pc.order;
   std::vector<double> cw;
@@ -254,122 +293,120 @@ ufg_status wce_b(Batch& B, int prec, const void* r, void* z, bool tr,
   // order 2 in the momentum basis: the terms y0 (V.spec) and y1 (V.acc, unused there) are kept
   // and the last recurrence forms z = c0 y0 + c1 y1 + c2 y2 (no accumulator read-modify-write)
   const bool keep_terms = B.mom && d == 2;
-  for (auto& g : B.groups) {
-    const void* bk = prec ? (const void*)g.lat->bk32 : (const void*)g.lat->bk64;
-    if (keep_terms) {
-      if (!slice_m1w_supported(g.lat->nx, prec))
-        return cuda_fail(cudaErrorInvalidValue, "momentum-basis WCE");
-      auto recb = [&](const void* in, void* out, int mode, double coef) -> ufg_status {
-        note_launches(1);
-        KTimer kt(std::string("recurrence ") + (mode == 3 ? "sum3" : "out") +
-                      (prec ? " f32" : " f64"),
-                  B.st, batch_work(B, &g.probs, 0, (prec ? 4.0 : 8.0) * (mode == 3 ? 4 : 2)));
-        cudaError_t e = launch_recurrence_batch(
-            prec, in, out, bk, g.max_ntau, tr ? 1 : 0, 1.0, mode == 3 ? z : nullptr, coef, mode, 0,
-            g.rtiles, g.nrtiles, B.probs, B.st, V.spec, V.acc, cw[0], cw[1]);
-        if (e != cudaSuccess) return cuda_fail(e, "batched recurrence");
-        return UFG_OK;
-      };
-      auto m1 = [&](const void* in) -> ufg_status {  // -A M1 (or M1^T) in momentum space
-        SliceCall m = base_call(g.lat, FAM_INV, prec);
-        m.fam = FAM_M1W;
-        m.coef2 = base_call(g.lat, FAM_FWD, prec).coef;
-        m.in = in;
-        m.pre = fldb(B, 's', prec);
-        if (tr) m.bkpre = bk; else m.bkpost = bk;
-        m.shift = tr ? +1 : -1;
-        m.a = -1.0;
-        m.scale_by_A = 1;
-        m.out = V.wr;
-        return slice(B, g, m, 0);
-      };
-      UFG_TRY(recb(r, V.spec, 0, 0.0));     // y0
-      UFG_TRY(m1(V.spec));
-      UFG_TRY(recb(V.wr, V.acc, 0, 0.0));   // y1
-      UFG_TRY(m1(V.acc));
-      UFG_TRY(recb(V.wr, nullptr, 3, cw[2]));  // z = c0 y0 + c1 y1 + c2 y2
-      continue;
-    }
-    auto rec = [&](const void* in, double coef, int mode, bool write_out) -> ufg_status {
+  const void* bk = prec ? (const void*)g.lat->bk32 : (const void*)g.lat->bk64;
+  if (keep_terms) {
+    if (!slice_m1w_supported(g.lat->nx, prec))
+      return cuda_fail(cudaErrorInvalidValue, "momentum-basis WCE");
+    auto recb = [&](const void* in, void* out, int mode, double coef) -> ufg_status {
       note_launches(1);
-      KTimer kt(std::string("recurrence acc") + std::to_string(mode) + (write_out ? "+out" : "") +
+      KTimer kt(std::string("recurrence ") + (mode == 3 ? "sum3" : "out") +
                     (prec ? " f32" : " f64"),
-                B.st,
-                batch_work(B, &g.probs, 0,
-                           (prec ? 4.0 : 8.0) *
-                               (1 + (mode == 1 ? 1 : mode == 2 ? 2 : 0) + (write_out ? 1 : 0))));
-      cudaError_t e = launch_recurrence_batch(prec, in, write_out ? V.spec : nullptr, bk,
-                                              g.max_ntau, tr ? 1 : 0, 1.0, acc, coef, mode, 0,
-                                              g.rtiles, g.nrtiles, B.probs, B.st);
+                B.gs, batch_work(B, &g.probs, 0, (prec ? 4.0 : 8.0) * (mode == 3 ? 4 : 2)));
+      cudaError_t e = launch_recurrence_batch(
+          prec, in, out, bk, g.max_ntau, tr ? 1 : 0, 1.0, mode == 3 ? z : nullptr, coef, mode, 0,
+          g.rtiles, g.nrtiles, B.probs, B.gs, V.spec, V.acc, cw[0], cw[1]);
       if (e != cudaSuccess) return cuda_fail(e, "batched recurrence");
       return UFG_OK;
     };
-    if (B.mom) {
-      UFG_TRY(rec(r, cw[0], 1, d > 0));
-    } else {
-      SliceCall fw = base_call(g.lat, FAM_FWD, prec);
-      fw.in = r;
-      fw.out = V.spec;
-      if (prep_r != nullptr) {
-        fw.prep_r = prep_r;
-        fw.prep_v = prep_v;
-        fw.prep_out = const_cast<void*>(r);
-      }
-      UFG_TRY(slice(B, g, fw, 0));
-      UFG_TRY(rec(V.spec, cw[0], 1, d > 0));
+    auto m1 = [&](const void* in) -> ufg_status {  // -A M1 (or M1^T) in momentum space
+      SliceCall m = base_call(g.lat, FAM_INV, prec);
+      m.fam = FAM_M1W;
+      m.coef2 = base_call(g.lat, FAM_FWD, prec).coef;
+      m.in = in;
+      m.pre = fldb(B, 's', prec);
+      if (tr) m.bkpre = bk; else m.bkpost = bk;
+      m.shift = tr ? +1 : -1;
+      m.a = -1.0;
+      m.scale_by_A = 1;
+      m.out = V.wr;
+      return slice(B, g, m, 0);
+    };
+    UFG_TRY(recb(r, V.spec, 0, 0.0));     // y0
+    UFG_TRY(m1(V.spec));
+    UFG_TRY(recb(V.wr, V.acc, 0, 0.0));   // y1
+    UFG_TRY(m1(V.acc));
+    UFG_TRY(recb(V.wr, nullptr, 3, cw[2]));  // z = c0 y0 + c1 y1 + c2 y2
+    return UFG_OK;
+  }
+  auto rec = [&](const void* in, double coef, int mode, bool write_out) -> ufg_status {
+    note_launches(1);
+    KTimer kt(std::string("recurrence acc") + std::to_string(mode) + (write_out ? "+out" : "") +
+                  (prec ? " f32" : " f64"),
+              B.gs,
+              batch_work(B, &g.probs, 0,
+                         (prec ? 4.0 : 8.0) *
+                             (1 + (mode == 1 ? 1 : mode == 2 ? 2 : 0) + (write_out ? 1 : 0))));
+    cudaError_t e = launch_recurrence_batch(prec, in, write_out ? V.spec : nullptr, bk,
+                                            g.max_ntau, tr ? 1 : 0, 1.0, acc, coef, mode, 0,
+                                            g.rtiles, g.nrtiles, B.probs, B.gs);
+    if (e != cudaSuccess) return cuda_fail(e, "batched recurrence");
+    return UFG_OK;
+  };
+  if (B.mom) {
+    UFG_TRY(rec(r, cw[0], 1, d > 0));
+  } else {
+    SliceCall fw = base_call(g.lat, FAM_FWD, prec);
+    fw.in = r;
+    fw.out = V.spec;
+    if (prep_r != nullptr) {
+      fw.prep_r = prep_r;
+      fw.prep_v = prep_v;
+      fw.prep_out = const_cast<void*>(r);
     }
-    const bool fused = slice_m1w_supported(g.lat->nx, prec);
-    if (B.mom && !fused) return cuda_fail(cudaErrorInvalidValue, "momentum-basis WCE");
-    for (int nn = 1; nn <= d; ++nn) {
-      if (fused) {  // -A M1 (or M1^T) in momentum space in one kernel: spec -> wr
-        SliceCall m = base_call(g.lat, FAM_INV, prec);
-        m.fam = FAM_M1W;
-        m.coef2 = base_call(g.lat, FAM_FWD, prec).coef;
-        m.in = V.spec;
-        m.pre = fldb(B, 's', prec);
-        if (tr) m.bkpre = bk; else m.bkpost = bk;
-        m.shift = tr ? +1 : -1;
-        m.a = -1.0;
-        m.scale_by_A = 1;
-        m.out = V.wr;
-        UFG_TRY(slice(B, g, m, 0));
-      } else if (!tr) {
-        SliceCall iv = base_call(g.lat, FAM_INV, prec);
-        iv.in = V.spec;
-        iv.out = V.wr;
-        UFG_TRY(slice(B, g, iv, 0));
-        SliceCall m1 = base_call(g.lat, FAM_FWD, prec);
-        m1.in = V.wr;
-        m1.pre = fldb(B, 's', prec);
-        m1.bkpost = bk;
-        m1.shift = -1;
-        m1.a = -1.0;
-        m1.scale_by_A = 1;
-        m1.out = V.spec;
-        UFG_TRY(slice(B, g, m1, 0));
-      } else {
-        SliceCall m1t = base_call(g.lat, FAM_INV, prec);
-        m1t.in = V.spec;
-        m1t.bkpre = bk;
-        m1t.post = fldb(B, 's', prec);
-        m1t.shift = +1;
-        m1t.a = -1.0;
-        m1t.scale_by_A = 1;
-        m1t.out = V.wr;
-        UFG_TRY(slice(B, g, m1t, 0));
-        SliceCall fw2 = base_call(g.lat, FAM_FWD, prec);
-        fw2.in = V.wr;
-        fw2.out = V.spec;
-        UFG_TRY(slice(B, g, fw2, 0));
-      }
-      UFG_TRY(rec(fused ? V.wr : V.spec, cw[nn], 2, nn < d));
-    }
-    if (!B.mom) {
+    UFG_TRY(slice(B, g, fw, 0));
+    UFG_TRY(rec(V.spec, cw[0], 1, d > 0));
+  }
+  const bool fused = slice_m1w_supported(g.lat->nx, prec);
+  if (B.mom && !fused) return cuda_fail(cudaErrorInvalidValue, "momentum-basis WCE");
+  for (int nn = 1; nn <= d; ++nn) {
+    if (fused) {  // -A M1 (or M1^T) in momentum space in one kernel: spec -> wr
+      SliceCall m = base_call(g.lat, FAM_INV, prec);
+      m.fam = FAM_M1W;
+      m.coef2 = base_call(g.lat, FAM_FWD, prec).coef;
+      m.in = V.spec;
+      m.pre = fldb(B, 's', prec);
+      if (tr) m.bkpre = bk; else m.bkpost = bk;
+      m.shift = tr ? +1 : -1;
+      m.a = -1.0;
+      m.scale_by_A = 1;
+      m.out = V.wr;
+      UFG_TRY(slice(B, g, m, 0));
+    } else if (!tr) {
       SliceCall iv = base_call(g.lat, FAM_INV, prec);
-      iv.in = V.acc;
-      iv.out = z;
+      iv.in = V.spec;
+      iv.out = V.wr;
       UFG_TRY(slice(B, g, iv, 0));
+      SliceCall m1 = base_call(g.lat, FAM_FWD, prec);
+      m1.in = V.wr;
+      m1.pre = fldb(B, 's', prec);
+      m1.bkpost = bk;
+      m1.shift = -1;
+      m1.a = -1.0;
+      m1.scale_by_A = 1;
+      m1.out = V.spec;
+      UFG_TRY(slice(B, g, m1, 0));
+    } else {
+      SliceCall m1t = base_call(g.lat, FAM_INV, prec);
+      m1t.in = V.spec;
+      m1t.bkpre = bk;
+      m1t.post = fldb(B, 's', prec);
+      m1t.shift = +1;
+      m1t.a = -1.0;
+      m1t.scale_by_A = 1;
+      m1t.out = V.wr;
+      UFG_TRY(slice(B, g, m1t, 0));
+      SliceCall fw2 = base_call(g.lat, FAM_FWD, prec);
+      fw2.in = V.wr;
+      fw2.out = V.spec;
+      UFG_TRY(slice(B, g, fw2, 0));
     }
+    UFG_TRY(rec(fused ? V.wr : V.spec, cw[nn], 2, nn < d));
+  }
+  if (!B.mom) {
+    SliceCall iv = base_call(g.lat, FAM_INV, prec);
+    iv.in = V.acc;
+    iv.out = z;
+    UFG_TRY(slice(B, g, iv, 0));
   }
   return UFG_OK;
 }
@@ -438,22 +475,20 @@ ufg_status bicg_b(Batch& B, int prec, int op, const std::vector<double>& tol,
   auto body = [&]() -> ufg_status {
     if (!fuse_p)
       UFG_TRY(vecb(B, prec, V_BI_P, 0, V.p, V.r, V.v, nullptr, nullptr, nullptr, nullptr));
-    const void* y = V.p;
-    if (pc) {
-      UFG_TRY(wce_b(B, prec, V.p, V.y, tr, fuse_p ? V.r : nullptr, V.v));
-      y = V.y;
-    }
-    UFG_TRY(apply_b(B, prec, op, y, V.v, 1.0, nullptr, 0.0, V.rhat, false, B.slot(B_SLICE1), 0,
-                    OP_BI_ALPHA));
+    const void* y = pc ? V.y : V.p;
+    UFG_TRY(for_groups(B, [&](Group& g) -> ufg_status {
+      if (pc) UFG_TRY(wce_g(B, g, prec, V.p, V.y, tr, fuse_p ? V.r : nullptr, V.v));
+      return apply_g(B, g, prec, op, y, V.v, 1.0, nullptr, 0.0, V.rhat, false,
+                     B.slot(B_SLICE1), 0, OP_BI_ALPHA);
+    }));
     UFG_TRY(vecb(B, prec, V_BI_S, 0, V.s, V.r, V.v, V.x, y, nullptr, B.slot(B_VEC1),
                  OP_BI_SCHECK));
-    const void* z = V.s;
-    if (pc) {
-      UFG_TRY(wce_b(B, prec, V.s, V.z, tr));
-      z = V.z;
-    }
-    UFG_TRY(apply_b(B, prec, op, z, V.t, 1.0, nullptr, 0.0, V.s, true, B.slot(B_SLICE2), 0,
-                    OP_BI_OMEGA));
+    const void* z = pc ? V.z : V.s;
+    UFG_TRY(for_groups(B, [&](Group& g) -> ufg_status {
+      if (pc) UFG_TRY(wce_g(B, g, prec, V.s, V.z, tr));
+      return apply_g(B, g, prec, op, z, V.t, 1.0, nullptr, 0.0, V.s, true, B.slot(B_SLICE2), 0,
+                     OP_BI_OMEGA);
+    }));
     UFG_TRY(vecb(B, prec, V_BI_X, 0, V.x, z, V.r, V.s, V.t, V.rhat, B.slot(B_VEC2),
                  OP_BI_RCHECK_RHO));
     return UFG_OK;
@@ -811,13 +846,12 @@ ufg_status solve_in_basis(Batch& B, int op, const double* rhs, double* x,
 
 // y = F x (inverse: F^T x) per slice for every problem, FP64 arenas
 ufg_status fourier_b(Batch& B, const double* x, double* y, bool inverse) {
-  for (auto& g : B.groups) {
+  return for_groups(B, [&](Group& g) {
     SliceCall c = base_call(g.lat, inverse ? FAM_INV : FAM_FWD, 0);
     c.in = x;
     c.out = y;
-    UFG_TRY(slice(B, g, c, -1));
-  }
-  return UFG_OK;
+    return slice(B, g, c, -1);
+  });
 }
 
 // Whether the batch solves in the momentum basis: with the WCE preconditioner, whose forward and
@@ -983,6 +1017,7 @@ ufg_status setup(Batch& B, int n, const ufg_problem* probs) {
   B.n = n;
   B.pr.assign(probs, probs + n);
   UFG_CUDA(cudaStreamCreateWithFlags(&B.st, cudaStreamNonBlocking));
+  B.gs = B.st;
   // order problems by size (largest first) inside the arenas and tile tables
   std::vector<int> order(n);
   for (int i = 0; i < n; ++i) order[i] = i;
@@ -1015,6 +1050,16 @@ ufg_status setup(Batch& B, int n, const ufg_problem* probs) {
     }
     B.groups[gi].probs.push_back(i);
     B.group_of[i] = gi;
+  }
+  constexpr size_t MAX_BRANCHES = 8;  // streams in all, whatever the number of groups
+  for (size_t i = 0; i < std::min(B.groups.size(), MAX_BRANCHES) && B.groups.size() > 1; ++i) {
+    cudaEvent_t ev = nullptr;
+    UFG_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+    B.fork_ev.push_back(ev);
+    if (i == 0) continue;
+    cudaStream_t fs = nullptr;
+    UFG_CUDA(cudaStreamCreateWithFlags(&fs, cudaStreamNonBlocking));
+    B.fork_st.push_back(fs);
   }
   B.probs_h.assign(n, BatchProb{});
   UFG_TRY(B.alloc(&B.scs, (size_t)n));
