@@ -299,7 +299,7 @@ ufg_status wce_g(Batch& B, Group& g, int prec, const void* r, void* z, bool tr,
       return cuda_fail(cudaErrorInvalidValue, "momentum-basis WCE");
     auto recb = [&](const void* in, void* out, int mode, double coef) -> ufg_status {
       note_launches(1);
-      KTimer kt(std::string("recurrence ") + (mode == 3 ? "sum3" : "out") +
+      KTimer kt(std::string("recurrence ") + (mode == 3 ? "acc1+terms" : "out") +
                     (prec ? " f32" : " f64"),
                 B.gs, batch_work(B, &g.probs, 0, (prec ? 4.0 : 8.0) * (mode == 3 ? 4 : 2)));
       cudaError_t e = launch_recurrence_batch(
@@ -944,14 +944,11 @@ ufg_status build_slice_tiles(Batch& B, const ufg_problem* probs) {
   return UFG_OK;
 }
 
-// Time slices per slice tile, tuned per (N_x, tau) group whose slice kernels are the
-// shared-memory ones in FP32 (no TMA shape at this N_x; the TMA kernels take one slice per CTA):
-// at N_x = 6 a one-slice tile keeps 36 of 256 threads busy in a pass.  Each candidate (1, 2, 4, 8
+// Time slices per slice tile, tuned per (N_x, tau) group without a TMA shape (the TMA kernels
+// take one slice per CTA; at N_x = 8 a slice is two whole warps).  Each candidate (1, 2, 4, 8
 // slices within 48 KB of FP64 shared memory and the group's longest N_tau) is timed on the
-// batch's own arenas with the FP32 M apply, where mixed solves spend their time (with the FP64
-// apply in the sum the 96-problem batch chose one slice at N_x = 10 and 12 and took 78.9 instead
-// of 74.5 ms), on zeroed operands, three launches each after one; the fastest is kept
-// (ufg_stats.tile_slices).
+// batch's own arenas with the FP32 momentum-space M, where mixed solves spend their time, on
+// zeroed operands, three launches each after one; the fastest is kept (ufg_stats.tile_slices).
 ufg_status tune_tiles(Batch& B, const ufg_problem* probs) {
   auto tma_shape = [](int N, int prec) { return prec ? (N == 16 || N == 32) : (N == 8 || N == 16); };
   bool changed = false, zeroed = false;
@@ -982,10 +979,13 @@ ufg_status tune_tiles(Batch& B, const ufg_problem* probs) {
     for (int spc : cand) {
       g.spc = spc;
       if ((result = build_slice_tiles(B, probs)) != UFG_OK) break;
-      SliceCall c = base_call(g.lat, FAM_KIN, 1);
+      SliceCall c = base_call(g.lat, FAM_INV, 1);
+      c.fam = FAM_M1W;
+      c.coef2 = base_call(g.lat, FAM_FWD, 1).coef;
+      c.m1w_full = 1;
       c.in = B.ar[1].x;
       c.pre = B.w32;
-      c.id = c.in;
+      c.bkpost = g.lat->bk32;
       c.shift = -1;
       c.out = B.ar[1].t;
       if ((result = slice(B, g, c, -1)) != UFG_OK) break;  // warm-up

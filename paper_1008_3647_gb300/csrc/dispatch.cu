@@ -13,7 +13,8 @@ bool slice_supported_n(int N) {
 }
 
 bool slice_m1w_supported(int N, int prec) {
-  return prec == 1 ? N == 16 : (N == 8 || N == 16);
+  (void)prec;
+  return N < 32 && slice_supported_n(N);
 }
 
 bool slice_q_supported(int N, int prec, int ntau, int dim) {

@@ -739,7 +739,8 @@ ufg_status ufg_apply_M_momentum(ufg_field* f, const void* x, void* y, int prec, 
   if (prec == UFG_FP64_EMULATED) prec = UFG_FP64;
   UFG_TRY(check_vec(f, x, y, prec));
   const ufg_lattice* lat = f->lat;
-  if (lat->dim != 3 || !slice_m1w_supported(lat->nx, prec)) {
+  // (the solvers also use the kernels of the other extents)
+  if (lat->dim != 3 || !(lat->nx == 16 || (lat->nx == 8 && prec == UFG_FP64))) {
     set_error("momentum-space apply built for FP32 N_x = 16 and FP64 N_x = 8, 16 (got N_x = %d)",
               lat->nx);
     return UFG_INVALID_ARG;

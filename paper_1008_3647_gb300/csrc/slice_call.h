@@ -107,8 +107,8 @@ bool slice_tma_prep_supported(int N, int prec, int allow_tma);
 // Runtime dispatch over the supported N (4, 6, 8, 10, 12, 16, 32).
 cudaError_t slice_dispatch(int N, const SliceCall& c, cudaStream_t st);
 bool slice_supported_n(int N);
-// Whether the fused FAM_M1W kernel exists for (N, precision): one CTA per slice with the slice
-// in 64- or 128-byte TMA rows (FP32 N = 16, FP64 N = 8 and 16).
+// Whether the fused FAM_M1W kernel exists for (N, precision): every extent whose slice one CTA
+// holds.
 bool slice_m1w_supported(int N, int prec);
 // Whether the fused FAM_Q kernel runs for (N, precision, N_tau): N = 16 (FP32 and FP64),
 // 3 <= N_tau <= twice the SM count, TMA enabled and UFG_NO_FUSED_Q unset.

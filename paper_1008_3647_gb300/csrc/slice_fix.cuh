@@ -466,10 +466,10 @@ slice_fix_m1w_kernel(const __grid_constant__ FixM1wArgs<N> A) {
 // ---- launchers -------------------------------------------------------------------------------
 template <int N, class Args>
 inline void fix_common(Args& a, const SliceCall& c, cudaStream_t st) {
-  a.in = static_cast<const double*>(c.in);
-  a.out = static_cast<double*>(c.out);
-  a.U = static_cast<const double*>(c.U);
-  a.dotP = static_cast<const double*>(c.dotP);
+  a.in = static_cast<decltype(a.in)>(c.in);
+  a.out = static_cast<decltype(a.out)>(c.out);
+  a.U = static_cast<decltype(a.U)>(c.U);
+  a.dotP = static_cast<decltype(a.dotP)>(c.dotP);
   a.a = c.a;
   a.bU = c.bU;
   a.partials = c.partials;
@@ -491,8 +491,8 @@ inline void fix_common(Args& a, const SliceCall& c, cudaStream_t st) {
   a.expire = (c.allow_tma && c.err != nullptr && (N == 8 || N == 16)) ? take_expired_wait(st) : 0;
 }
 
-// the launch of a kernel of this file: spc slices per CTA (cluster)
-template <int N, class Args>
+// the launch of a kernel on this plan: spc slices per CTA (cluster), shared words of type W
+template <int N, class W, class Args>
 inline cudaError_t fix_launch(void (*kern)(Args), int* configured, const Args& a,
                               const SliceCall& c, cudaStream_t st) {
   using S = FixShape<N>;
@@ -504,7 +504,7 @@ inline cudaError_t fix_launch(void (*kern)(Args), int* configured, const Args& a
   if (!*configured) {
     cudaError_t e =
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(S::MAXS * S::SLOT * sizeof(long long)));
+                             (int)(S::MAXS * S::SLOT * sizeof(W)));
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared);
@@ -514,7 +514,7 @@ inline cudaError_t fix_launch(void (*kern)(Args), int* configured, const Args& a
   const int units = c.tiles != nullptr ? c.ntiles : (c.ntau + a.spc - 1) / a.spc;
   if (c.grid_out) *c.grid_out = units * S::C;
   return launch_k(kern, dim3(units * S::C), dim3(a.spc * S::TS),
-                  (size_t)a.spc * S::SLOT * sizeof(long long), st, S::C, a);
+                  (size_t)a.spc * S::SLOT * sizeof(W), st, S::C, a);
 }
 
 template <int N, int FAM, int EPI>
@@ -533,7 +533,7 @@ inline cudaError_t fix_launch_epi(const SliceCall& c, cudaStream_t st) {
   a.cV = c.cV;
   a.shift = c.shift;
   static int configured = 0;
-  return fix_launch<N>(slice_fix_kernel<N, FAM, EPI>, &configured, a, c, st);
+  return fix_launch<N, long long>(slice_fix_kernel<N, FAM, EPI>, &configured, a, c, st);
 }
 
 template <int N>
@@ -583,7 +583,7 @@ inline cudaError_t fix_m1w_launch(const SliceCall& c, cudaStream_t st) {
   a.bk = static_cast<const double*>(DIR == 1 ? c.bkpre : c.bkpost);
   a.full_scale = c.full_scale;
   static int configured = 0;
-  return fix_launch<N>(slice_fix_m1w_kernel<N, DIR, FULL>, &configured, a, c, st);
+  return fix_launch<N, long long>(slice_fix_m1w_kernel<N, DIR, FULL>, &configured, a, c, st);
 }
 
 // FP64 slice launch of a 3-D lattice.

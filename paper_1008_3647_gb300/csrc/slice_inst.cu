@@ -7,6 +7,7 @@
 #include "slice_pair.cuh"
 #include "slice_lowd.cuh"
 #include "slice_q.cuh"
+#include "slice_reg.cuh"
 #include "slice_tma.cuh"
 
 #ifndef UFG_N
@@ -30,7 +31,8 @@ cudaError_t slice_launch<UFG_N>(const SliceCall& c, cudaStream_t st) {
   if (c.dim != 3) return slice_lowd_try<UFG_N>(c, st);       // 1-D and 2-D lattices
   if (c.prec == 0)  // the integer-pipe kernels, but for the 32^3 calls that keep the FP64 pipe
     return c.fp64_pipe ? slice_launch_fp64<UFG_N>(c, st) : slice_fix_try<UFG_N>(c, st);
-  if (c.fam == FAM_M1W) return slice_m1w_try<UFG_N>(c, st);  // callers check support first
+  if (c.fam == FAM_M1W)  // callers check support first; the staged form where it is faster
+    return UFG_N == 16 ? slice_m1w_try<UFG_N>(c, st) : slice_reg_m1w_try<UFG_N>(c, st);
   if (c.fam == FAM_Q) return slice_q_try<UFG_N>(c, st);      // callers check support first
   if (c.allow_tma && tma_enabled()) {
     const cudaError_t e = slice_tma_try<UFG_N>(c, st);
