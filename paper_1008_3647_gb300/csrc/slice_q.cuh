@@ -13,6 +13,11 @@
 // launch instead of two and no intermediate vector in memory: at 16^3 the two launches are
 // bound by latency (one CTA per slice, few CTAs per SM), not by their bytes.  The multiplier
 // rows of the x-passes come from global memory (16-byte loads), the epilogue's w_t per site.
+// Stages A and B run side by side in the two halves of the CTA, and the multiplier rows are
+// requested before the boxes arrive: back to back 13.3 -> 8.0 us at 16^3 x 256 with programmatic
+// dependent launch, which the solvers use for this kernel (CG + Chebyshev 16, mixed: 195 -> 183 us
+// per iteration of 17 Q; without it the launch gaps hid the gain).  Latency-bound: 256 CTAs on
+// 152 SMs, issue 27 %.
 // Built for FP32 16^3 slices; slice_q_supported says where it runs.
 #pragma once
 #include <cuda.h>
@@ -40,50 +45,60 @@ struct QArgs {
   const int* done;
   int exec_if;
   int ntau;
+  int fop;  // scalar op of the grid's last CTA (-1: none), see SliceCall
+  DevScalars* scs;
+  unsigned* counters;
   int* err;
   int expire;  // test hook, see TmaArgs
 };
 
-template <int N, typename R>
-constexpr int q_min_blocks() {
-  return 4;  // three boxes of one 16^3 slice: 48 KB
-}
+// Stages A and B (see above) share no output, so two halves of the CTA run them side by side: six
+// passes in a row instead of nine (x_t is loaded twice, once per half).
+constexpr int Q_NT = 2 * TMA_NT;
 
-// x-pass in place: rows of X (times the multiplier rows of wg when given)
-template <int N, typename R, class CF>
-__device__ __forceinline__ void q_xpass(R* X, const R* __restrict__ wg, const CF& cf) {
+// x-pass in place, row r: times the multiplier row w when MUL
+template <int N, typename R, bool MUL, class CF>
+__device__ __forceinline__ void q_xpass(R* X, int r, const R (&w)[N], const CF& cf) {
   using G = SwzGeom<N, R>;
   constexpr int CPR = G::RB / 16, EPC = 16 / (int)sizeof(R);
-  for (int r = threadIdx.x; r < N * N; r += TMA_NT) {
-    R v[N];
+  R v[N];
 #pragma unroll
-    for (int c = 0; c < CPR; ++c) {
-      const int o = G::chunk(r, c);
-      R vc[EPC];
+  for (int c = 0; c < CPR; ++c) {
+    const int o = G::chunk(r, c);
+    R vc[EPC], wc[EPC];
 #pragma unroll
-      for (int e = 0; e < EPC; ++e) vc[e] = X[o + e];
-      if (wg != nullptr) {
-        R wc[EPC];
-        ld16(wg + r * N + c * EPC, wc);
-        mul_chunk(vc, wc);
-      }
-#pragma unroll
-      for (int e = 0; e < EPC; ++e) v[c * EPC + e] = vc[e];
+    for (int e = 0; e < EPC; ++e) {
+      vc[e] = X[o + e];
+      wc[e] = w[c * EPC + e];
     }
-    swz_store_row<N, R>(X, r, v, cf, false, false);
+    if constexpr (MUL) mul_chunk(vc, wc);
+#pragma unroll
+    for (int e = 0; e < EPC; ++e) v[c * EPC + e] = vc[e];
   }
+  swz_store_row<N, R>(X, r, v, cf, false, false);
+}
+
+// y-pass in place, column l = (plane, x)
+template <int N, typename R, class CF>
+__device__ __forceinline__ void q_ypass(R* X, int l, const CF& cf) {
+  using G = SwzGeom<N, R>;
+  const int p = l / N, x = l - (l / N) * N;
+  R v[N];
+#pragma unroll
+  for (int y = 0; y < N; ++y) v[y] = X[G::off(p * N + y, x)];
+  line_op<N, R, false, false>(v, cf, [&](int i, R val) { X[G::off(p * N + i, x)] = val; });
 }
 
 template <int N, typename R, bool UV, bool DOT>
-__global__ void __launch_bounds__(TMA_NT, (q_min_blocks<N, R>()))
+__global__ void __launch_bounds__(Q_NT, 2)
 slice_q_kernel(const __grid_constant__ QArgs<N, R> A) {
   pdl_begin();
   using G = SwzGeom<N, R>;
   constexpr int NN = N * N;
   constexpr int VOL = N * NN;
-  static_assert(NN <= TMA_NT, "one row, line and column per thread and pass");
+  static_assert(NN == TMA_NT, "one row, line and column per thread of a half");
   extern __shared__ __align__(1024) unsigned char tma_smem[];
-  __shared__ double red[TMA_NT / 32][2];
+  __shared__ double red[Q_NT / 32][2];
   __shared__ alignas(8) uint64_t bar, bar2;
   const int tid = threadIdx.x;
   const int t = blockIdx.x;
@@ -98,60 +113,66 @@ slice_q_kernel(const __grid_constant__ QArgs<N, R> A) {
   R* const X0 = reinterpret_cast<R*>(base);
   R* const X1 = X0 + VOL;
   R* const X2 = X1 + VOL;
+  R* const X3 = X2 + VOL;  // x_t again, for stage A's epilogue
   if (tid == 0) {
     mbar_init(&bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    mbar_expect_tx(&bar, (uint32_t)(3 * VOL * sizeof(R)));
+    mbar_expect_tx(&bar, (uint32_t)(4 * VOL * sizeof(R)));
     tma_load_rows(X0, &A.tm_in, tm * NN, &bar);
     tma_load_rows(X1, &A.tm_in, t * NN, &bar);
     tma_load_rows(X2, &A.tm_in, tp * NN, &bar);
+    tma_load_rows(X3, &A.tm_in, t * NN, &bar);
+  }
+  // this thread's multiplier row of its first x-pass, while the boxes are in flight
+  const R* const w_tm = A.w + (size_t)tm * VOL;
+  const R* const w_t = A.w + (size_t)t * VOL;
+  R wrow[N];
+  {
+    constexpr int EPC = 16 / (int)sizeof(R);
+    const R* src = (tid >= NN ? w_t + (size_t)(tid - NN) * N : w_tm + (size_t)tid * N);
+#pragma unroll
+    for (int c = 0; c < N / EPC; ++c) {
+      R w4[EPC];
+      ld16(src + c * EPC, w4);
+#pragma unroll
+      for (int e = 0; e < EPC; ++e) wrow[c * EPC + e] = w4[e];
+    }
   }
   __syncthreads();
   mbar_wait_bounded(&bar, 0u, TMA_WAIT_LIMIT, A.err);
   if (A.expire && tid == 0) mbar_expire_one_wait(&bar2, EXPIRE_LIMIT, A.err);
-  const R* const w_tm = A.w + (size_t)tm * VOL;
-  const R* const w_t = A.w + (size_t)t * VOL;
-  // ---- A: X0 <- x_t + sm(t) T(w_{t-1} x_{t-1}) ----
-  q_xpass<N, R>(X0, w_tm, A.cx);
-  __syncthreads();
-  swz_ypass<N, R, false, false>(X0, A.cy);
-  __syncthreads();
-  for (int q = tid; q < NN; q += TMA_NT) {
-    const int y = q / N, x = q - (q / N) * N;
+  // ---- A: X0 <- x_t + sm(t) T(w_{t-1} x_{t-1});  B: X2 <- x_{t+1} + sm(t+1) T(w_t x_t) ----
+  {
+    const bool second = tid >= NN;
+    const int l = second ? tid - NN : tid;
+    R* const X = second ? X1 : X0;
+    q_xpass<N, R, true>(X, l, wrow, A.cx);
+    __syncthreads();
+    q_ypass<N, R>(X, l, A.cy);
+    __syncthreads();
+    const R* const id = second ? X2 : X3;
+    R* const dst = second ? X2 : X0;
+    const R sg = second ? sB : sA;
+    const int y = l / N, x = l - (l / N) * N;
     R v[N];
 #pragma unroll
-    for (int z = 0; z < N; ++z) v[z] = X0[G::off(z * N + y, x)];
+    for (int z = 0; z < N; ++z) v[z] = X[G::off(z * N + y, x)];
     line_op<N, R, false, false>(v, A.cz, [&](int zp, R val) {
       const int o = G::off(zp * N + y, x);
-      X0[o] = fmadd(sA, val, X1[o]);
-    });
-  }
-  __syncthreads();
-  // ---- B: X2 <- x_{t+1} + sm(t+1) T(w_t x_t) ----
-  q_xpass<N, R>(X1, w_t, A.cx);
-  __syncthreads();
-  swz_ypass<N, R, false, false>(X1, A.cy);
-  __syncthreads();
-  for (int q = tid; q < NN; q += TMA_NT) {
-    const int y = q / N, x = q - (q / N) * N;
-    R v[N];
-#pragma unroll
-    for (int z = 0; z < N; ++z) v[z] = X1[G::off(z * N + y, x)];
-    line_op<N, R, false, false>(v, A.cz, [&](int zp, R val) {
-      const int o = G::off(zp * N + y, x);
-      X2[o] = fmadd(sB, val, X2[o]);
+      dst[o] = fmadd(sg, val, id[o]);
     });
   }
   __syncthreads();
   // ---- C: q_t = a (y_t + st(t) w_t T(y_{t+1})) + bU U + cV V ----
-  q_xpass<N, R>(X2, static_cast<const R*>(nullptr), A.cx);
+  if (tid < NN) q_xpass<N, R, false>(X2, tid, wrow, A.cx);
   __syncthreads();
-  swz_ypass<N, R, false, false>(X2, A.cy);
+  if (tid < NN) q_ypass<N, R>(X2, tid, A.cy);
   __syncthreads();
   const size_t obase0 = (size_t)t * VOL;
   const R ra = R(A.a), rbU = R(A.bU), rcV = R(A.cV);
   R acc_dot = R(0), acc_self = R(0);
-  for (int q = tid; q < NN; q += TMA_NT) {
+  if (tid < NN) {
+    const int q = tid;
     const int y = q / N, x = q - (q / N) * N;
     R v[N];
 #pragma unroll
@@ -186,13 +207,14 @@ slice_q_kernel(const __grid_constant__ QArgs<N, R> A) {
     __syncthreads();
     if (tid == 0) {
       double d = 0.0, q2 = 0.0;
-      for (int wi = 0; wi < TMA_NT / 32; ++wi) {
+      for (int wi = 0; wi < Q_NT / 32; ++wi) {
         d += red[wi][0];
         q2 += red[wi][1];
       }
       A.partials[2 * blockIdx.x] = d;
       A.partials[2 * blockIdx.x + 1] = q2;
     }
+    if (A.fop >= 0) last_block_update_any(A.fop, A.scs, A.partials, 0, (int)gridDim.x, A.counters);
   }
 }
 
@@ -203,7 +225,8 @@ inline cudaError_t q_launch(const SliceCall& c, cudaStream_t st) {
   std::memset(&a, 0, sizeof(a));
   if (c.in == nullptr || c.pre == nullptr || c.out == nullptr || c.coef == nullptr ||
       c.ntau < 3 || c.tiles != nullptr || (c.want_dotP && c.dotP == nullptr) ||
-      ((c.want_dotP || c.want_self) && c.partials == nullptr))
+      ((c.want_dotP || c.want_self) && c.partials == nullptr) ||
+      (c.fop >= 0 && (!DOT || c.scs == nullptr || c.counters == nullptr)))
     return cudaErrorInvalidValue;
   if (encode_rows<R>(&a.tm_in, c.in, (long long)c.ntau * VOL, N, N * N) != cudaSuccess)
     return cudaErrorNotSupported;
@@ -224,9 +247,12 @@ inline cudaError_t q_launch(const SliceCall& c, cudaStream_t st) {
   a.done = c.done;
   a.exec_if = c.exec_if;
   a.ntau = c.ntau;
+  a.fop = c.fop;
+  a.scs = c.scs;
+  a.counters = c.counters;
   a.err = c.err;
   a.expire = take_expired_wait(st);
-  const size_t smem = 3 * (size_t)VOL * sizeof(R) + 1024;
+  const size_t smem = 4 * (size_t)VOL * sizeof(R) + 1024;
   auto kern = slice_q_kernel<N, R, UV, DOT>;
   static int configured = 0;
   if (!configured) {
@@ -239,7 +265,7 @@ inline cudaError_t q_launch(const SliceCall& c, cudaStream_t st) {
     configured = 1;
   }
   if (c.grid_out) *c.grid_out = c.ntau;
-  return launch_k(kern, dim3(c.ntau), dim3(TMA_NT), smem, st, 1, a);
+  return launch_k(kern, dim3(c.ntau), dim3(Q_NT), smem, st, 1, a);
 }
 
 template <int N, typename R>
