@@ -41,16 +41,8 @@ int vec_grid(long long n) {
 
 __device__ __forceinline__ void block_pair_store(double d1, double d2, double* part) {
   __shared__ double red[VEC_NT / 32][2];
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    d1 += __shfl_xor_sync(0xffffffffu, d1, off);
-    d2 += __shfl_xor_sync(0xffffffffu, d2, off);
-  }
-  const int w = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) {
-    red[w][0] = d1;
-    red[w][1] = d2;
-  }
+  const double v = warp_sum2(d1, d2);
+  if ((threadIdx.x & 15) == 0) red[threadIdx.x >> 5][(threadIdx.x >> 4) & 1] = v;
   __syncthreads();
   if (threadIdx.x == 0) {
     double a = 0.0, b = 0.0;

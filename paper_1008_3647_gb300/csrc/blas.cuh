@@ -34,6 +34,7 @@ enum ScalarOp {
   OP_CG_ALPHA,      // alpha = rz / (p.q)
   OP_CG_CHECK,      // iters++, rr = r.r, converged?
   OP_CG_BETA,       // rz_new = r.z, beta = rz_new / rz
+  OP_CG_CHECK_BETA, // without preconditioner: the check and, still running, beta from the same r.r
   OP_BI_ALPHA,      // alpha = rho / (rhat.v)
   OP_BI_SCHECK,     // ss = s.s, converged?
   OP_BI_OMEGA,      // omega = (t.s) / (t.t)

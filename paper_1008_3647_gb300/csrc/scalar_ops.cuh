@@ -10,6 +10,18 @@ namespace ufg {
 
 constexpr int SCAL_NT = 256;  // threads of every CTA that runs these reductions
 
+// Sums of a and b over the warp with one addition per step after the first: lanes 0-15 go on with
+// a, lanes 16-31 with b (the pairing of the xor butterfly, so the sums keep their bits; an FP64
+// warp instruction takes 16 cycles of the SM's pipe).  a in lane 0, b in lane 16.
+static __device__ __forceinline__ double warp_sum2(double a, double b) {
+  const bool hi = (threadIdx.x & 16) != 0;
+  double v = hi ? b : a;
+  v += __shfl_xor_sync(0xffffffffu, hi ? a : b, 16);
+#pragma unroll
+  for (int off = 8; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  return v;
+}
+
 static __device__ __forceinline__ bool bad(double v) { return !isfinite(v); }
 
 // The four sums (pairs [i0, i1) of part, pairs [j0, j1) of part2) in one sweep: each thread adds
@@ -60,18 +72,31 @@ static __device__ __forceinline__ void bi_rho(DevScalars* sc, double rho, double
   if (bad(sc->beta)) sc->done = 4;
 }
 
+// |v| against a bound from v.v: no square root on the one thread's chain (FP64 divisions and roots
+// take hundreds of cycles here)
+static __device__ __forceinline__ bool within(double vv, double bound) { return vv <= bound * bound; }
+static __device__ __forceinline__ bool diverged(const DevScalars* sc, double vv) {
+  if (!(sc->div_limit > 0)) return false;
+  const double lim = sc->div_limit * sc->bn;
+  return vv > lim * lim;
+}
+
 static __device__ __forceinline__ void bi_rcheck(DevScalars* sc, double rr, double tb) {
   sc->rr = rr;
   sc->rho_old = sc->rho;
   if (bad(rr)) sc->done = 4;
-  else if (sqrt(rr) <= tb) sc->done = 1;
-  else if (sc->div_limit > 0 && sqrt(rr) > sc->div_limit * sc->bn) sc->done = 6;
+  else if (within(rr, tb)) sc->done = 1;
+  else if (diverged(sc, rr)) sc->done = 6;
   else if (sc->omega == 0.0) sc->done = 2;
   else if (sc->iters >= sc->maxit) sc->done = 5;
 }
 
-static __device__ __noinline__ void scalar_update(int op, DevScalars* sc, const double* part, double a0, double a1,
+// One thread.  The scalars are read at once, updated in registers and written back at once (read
+// where needed, each field was a dependent load from L2).
+static __device__ __noinline__ void scalar_update(int op, DevScalars* gsc, const double* part, double a0, double a1,
                               const double* part2, double b0, double b1) {
+  DevScalars local = *gsc;
+  DevScalars* const sc = &local;
   if ((op == OP_CG_INIT || op == OP_BI_INIT_RHO) && part2 != nullptr)
     sc->bn = sqrt(b1);  // rhs.rhs
   const double tb = sc->tol * sc->bn;
@@ -81,28 +106,32 @@ static __device__ __noinline__ void scalar_update(int op, DevScalars* sc, const 
       sc->rr = a1;
       sc->done = 0;
       if (bad(a0) || bad(a1)) sc->done = 4;
-      else if (sqrt(a1) <= tb) sc->done = 1;
+      else if (within(a1, tb)) sc->done = 1;
       break;
     case OP_CG_ALPHA:  // part = slice partials (p.q, -)
       sc->pq = a0;
       sc->alpha = sc->rz / a0;
       if (bad(sc->alpha)) sc->done = 4;
       break;
+    case OP_CG_CHECK_BETA:
     case OP_CG_CHECK:  // part = (-, r.r)
       sc->iters += 1;
       sc->rr = a1;
       if (bad(a1)) sc->done = 4;
-      else if (sqrt(a1) <= tb) sc->done = 1;
-      else if (sc->div_limit > 0 && sqrt(a1) > sc->div_limit * sc->bn) sc->done = 6;
+      else if (within(a1, tb)) sc->done = 1;
+      else if (diverged(sc, a1)) sc->done = 6;
       else if (sc->iters >= sc->maxit) sc->done = 5;
+      if (op == OP_CG_CHECK_BETA && sc->done == 0) {
+        sc->beta = a1 / sc->rz;
+        sc->rz = a1;
+        if (bad(sc->beta)) sc->done = 4;
+      }
       break;
-    case OP_CG_BETA: {  // part = (r.z, -) or, without preconditioner, part2 = (-, r.r)
-      const double rz_new = part != nullptr ? a0 : b1;
-      sc->beta = rz_new / sc->rz;
-      sc->rz = rz_new;
+    case OP_CG_BETA:  // part = (r.z, -)
+      sc->beta = a0 / sc->rz;
+      sc->rz = a0;
       if (bad(sc->beta)) sc->done = 4;
       break;
-    }
     case OP_BI_INIT_RHO:  // part = (rhat.r, r.r), part2 = (rhat.rhat, rhs.rhs); the first
                           // iteration's rho from the same partials
       sc->rho = a0;
@@ -113,7 +142,7 @@ static __device__ __noinline__ void scalar_update(int op, DevScalars* sc, const 
       sc->omega = 1.0;
       sc->done = 0;
       if (bad(a0) || bad(a1)) sc->done = 4;
-      else if (sqrt(a1) <= tb) sc->done = 1;
+      else if (within(a1, tb)) sc->done = 1;
       else bi_rho(sc, a0, a1);
       break;
     case OP_BI_RHO_REDO:  // part = (rhat.r, r.r) of the replaced residual
@@ -133,8 +162,8 @@ static __device__ __noinline__ void scalar_update(int op, DevScalars* sc, const 
     case OP_BI_SCHECK:  // part = (-, s.s)
       sc->ss = a1;
       if (bad(a1)) sc->done = 4;
-      else if (sqrt(a1) <= tb) sc->done = 1;
-      else if (sc->div_limit > 0 && sqrt(a1) > sc->div_limit * sc->bn) sc->done = 6;
+      else if (within(a1, tb)) sc->done = 1;
+      else if (diverged(sc, a1)) sc->done = 6;
       break;
     case OP_BI_OMEGA:  // part = slice partials (t.s, t.t)
       sc->omega = a1 > 0.0 ? a0 / a1 : 0.0;
@@ -149,6 +178,7 @@ static __device__ __noinline__ void scalar_update(int op, DevScalars* sc, const 
       if (sc->done == 0) bi_rho(sc, a0, a1);
       break;
   }
+  *gsc = local;
 }
 
 // Called by every thread of a CTA of a producer whose thread 0 has just written the CTA's
@@ -167,10 +197,22 @@ static __device__ __forceinline__ void last_block_update(int op, DevScalars* sc,
   __syncthreads();
   if (!is_last) return;
   __threadfence();
-  double r[4];
-  block_sums4<NT>(part, i0, i1, nullptr, 0, 0, r);
+  __shared__ double red[NT / 32][2];
+  double s0 = 0.0, s1 = 0.0;
+  for (int i = i0 + (int)threadIdx.x; i < i1; i += NT) {
+    s0 += part[2 * i];
+    s1 += part[2 * i + 1];
+  }
+  const double v = warp_sum2(s0, s1);
+  if ((threadIdx.x & 15) == 0) red[threadIdx.x >> 5][(threadIdx.x >> 4) & 1] = v;
+  __syncthreads();
   if (threadIdx.x == 0) {
-    scalar_update(op, sc, part, r[0], r[1], nullptr, 0.0, 0.0);
+    s0 = s1 = 0.0;
+    for (int w = 0; w < NT / 32; ++w) {
+      s0 += red[w][0];
+      s1 += red[w][1];
+    }
+    scalar_update(op, sc, part, s0, s1, nullptr, 0.0, 0.0);
     *counter = 0u;
   }
 }
@@ -195,15 +237,8 @@ static __device__ __forceinline__ void last_block_update_any(int op, DevScalars*
     s0 += part[2 * i];
     s1 += part[2 * i + 1];
   }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    s0 += __shfl_xor_sync(0xffffffffu, s0, off);
-    s1 += __shfl_xor_sync(0xffffffffu, s1, off);
-  }
-  if ((tid & 31) == 0) {
-    red[tid >> 5][0] = s0;
-    red[tid >> 5][1] = s1;
-  }
+  const double v = warp_sum2(s0, s1);
+  if ((tid & 15) == 0) red[tid >> 5][(tid >> 4) & 1] = v;
   __syncthreads();
   if (tid == 0) {
     s0 = s1 = 0.0;

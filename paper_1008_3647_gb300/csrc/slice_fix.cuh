@@ -205,15 +205,8 @@ __device__ __forceinline__ void fix_partials(double pd, double ps, double* parti
                                              unsigned* counters, int part_base) {
   __shared__ double red[32][2];
   const int tid = threadIdx.x, nw = (blockDim.x + 31) / 32;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    pd += __shfl_xor_sync(0xffffffffu, pd, o);
-    ps += __shfl_xor_sync(0xffffffffu, ps, o);
-  }
-  if ((tid & 31) == 0) {
-    red[tid >> 5][0] = pd;
-    red[tid >> 5][1] = ps;
-  }
+  const double v = warp_sum2(pd, ps);
+  if ((tid & 15) == 0) red[tid >> 5][(tid >> 4) & 1] = v;
   __syncthreads();
   if (tid == 0) {
     double d = 0.0, q = 0.0;

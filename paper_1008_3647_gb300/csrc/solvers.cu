@@ -120,18 +120,26 @@ SliceCall kin_call(const ufg_solver* S, const ufg_lattice* L, int prec) {
   return prec == 0 && S->fp64_pipe ? base_call_fp64(L) : base_call(L, FAM_KIN, prec);
 }
 
+// Whether the kernel that ends operator `op` carries the scalar step of its partials: the
+// momentum-space operator, the FP64 integer-pipe kernels and the fused Q.
+bool op_rides(const ufg_solver* S, const ufg_lattice* L, int prec, int op) {
+  if (S->mom) return true;
+  if (prec == 0) return L->dim == 3 && !kin_call(S, L, 0).fp64_pipe;
+  return op == OPK_Q && slice_q_supported(L->nx, prec, L->ntau, L->dim);
+}
+
 // ---- operator applications with epilogues --------------------------------------------------
 // out = a * (A in) + bU * U   with partials (out . dotP, out . out) into `part` when requested.
-// fop >= 0 (momentum basis only): the operator kernel's last CTA then applies scalar op fop to
-// the solver's scalars from those partials.
+// fop >= 0 (where op_rides): the operator kernel's last CTA then applies scalar op fop to the
+// solver's scalars from those partials.
 ufg_status apply_op(ufg_solver* S, const ufg_field* f, int prec, int op, const void* in, void* out,
                     double a, const void* U, double bU, const void* dotP, bool self, double* part,
                     int* nparts, int fop = -1) {
-  if (fop >= 0 && (!S->mom || part == nullptr)) {
-    set_error("fused scalar step requested outside the momentum-space operator");
+  const ufg_lattice* L = f->lat;
+  if (fop >= 0 && (!op_rides(S, L, prec, op) || part == nullptr)) {
+    set_error("fused scalar step requested of an operator kernel without one");
     return UFG_INTERNAL;
   }
-  const ufg_lattice* L = f->lat;
   const int* done = &S->sc->done;
   if (S->mom) {  // the fused momentum-space operator (BiCGStab only)
     if (op == OPK_Q) {
@@ -190,9 +198,18 @@ ufg_status apply_op(ufg_solver* S, const ufg_field* f, int prec, int op, const v
     c.want_self = self;
     c.partials = part;
     c.done = done;
+    if (fop >= 0) {
+      c.fop = fop;
+      c.scs = S->sc;
+      c.counters = S->fcount;
+    }
     int launched = 0;
     c.grid_out = &launched;
-    cudaError_t e = sdisp(L->nx, c, S->st);
+    cudaError_t e;
+    {
+      PdlScope pdl;
+      e = sdisp(L->nx, c, S->st);
+    }
     if (nparts) *nparts = launched;
     if (e != cudaSuccess) return cuda_fail(e, "fused Q kernel");
     S->counts.M++;
@@ -235,6 +252,11 @@ ufg_status apply_op(ufg_solver* S, const ufg_field* f, int prec, int op, const v
   c.want_self = self;
   c.partials = part;
   c.done = done;
+  if (fop >= 0) {
+    c.fop = fop;
+    c.scs = S->sc;
+    c.counters = S->fcount;
+  }
   int launched = 0;
   c.grid_out = &launched;
   cudaError_t e = sdisp(L->nx, c, S->st);
@@ -408,7 +430,7 @@ ufg_status pc_wce(ufg_solver* S, const ufg_field* f, int prec, const void* r, vo
     // order 2 in the momentum basis: the terms y0 (V.spec) and y1 (V.acc, unused there) are
     // kept and the last recurrence forms z = c0 y0 + c1 y1 + c2 y2
     auto recm = [&](const void* in, void* out, int mode) -> ufg_status {
-      KTimer kt(std::string("recurrence ") + (mode == 3 ? "sum3" : "out") + (prec ? " f32" : " f64"),
+      KTimer kt(std::string("recurrence ") + (mode == 3 ? "acc1+terms" : "out") + (prec ? " f32" : " f64"),
                 S->st, solo_work(done, 0, (double)L->S * (prec ? 4.0 : 8.0) * (mode == 3 ? 4 : 2)));
       cudaError_t er = launch_recurrence(prec, in, out, bk, L->V, L->ntau, tr ? 1 : 0, 1.0,
                                          mode == 3 ? z : nullptr, cw[2], mode, done, S->st, V.spec,
@@ -755,19 +777,18 @@ ufg_status run_cg(ufg_solver* S, ufg_field* f, int prec, double tol, int maxit, 
   VEC_NODONE(prec, V_COPY, n, V.p, z, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
   auto body = [&]() -> ufg_status {
     int nq = 0, nv = 0, npc = 0;
+    const bool ride = op_rides(S, f->lat, prec, OPK_Q);
     UFG_TRY(apply_op(S, f, prec, OPK_Q, V.p, V.q, 1.0, nullptr, 0.0, V.p, false, slot(S, P_SLICE1),
-                     &nq));
-    SCALAR(OP_CG_ALPHA, slot(S, P_SLICE1), nq, nullptr, 0);
-    // the residual check and (preconditioned) beta ride on the vector kernels that produce
-    // their partials: the last CTA applies the scalar step
+                     &nq, ride ? OP_CG_ALPHA : -1));
+    if (!ride) SCALAR(OP_CG_ALPHA, slot(S, P_SLICE1), nq, nullptr, 0);
+    // the residual check and beta ride on the vector kernels that produce their partials: the
+    // last CTA applies the scalar step
     VEC_SCALAR(prec, V_CG_UPDATE, n, V.x, V.p, V.r, V.q, nullptr, nullptr, slot(S, P_VEC1), &nv,
-               OP_CG_CHECK);
+               pc ? OP_CG_CHECK : OP_CG_CHECK_BETA);
     if (pc) {
       UFG_TRY(pc_apply_q(S, f, prec, V.r, V.z));
       VEC_SCALAR(prec, V_DOT, n, V.r, V.z, nullptr, nullptr, nullptr, nullptr, slot(S, P_PC),
                  &npc, OP_CG_BETA);
-    } else {
-      SCALAR(OP_CG_BETA, nullptr, 0, slot(S, P_VEC1), nv);
     }
     VEC(prec, V_CG_P, n, V.p, z, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
     return UFG_OK;
@@ -839,10 +860,11 @@ ufg_status run_bicgstab(ufg_solver* S, ufg_field* f, int prec, int op, double to
   };
   UFG_TRY(restart(x0));
   // The residual checks ride on the vector kernels that produce their partials (their last CTA
-  // applies the scalar step); alpha and omega, from the operator's partials, ride on the fused
-  // momentum-space operator and take scalar launches in the position basis.
+  // applies the scalar step); alpha and omega, from the operator's partials, ride on the operator
+  // kernel where it carries the step and take scalar launches elsewhere.
   auto body = [&]() -> ufg_status {
     int nsv = 0, nst = 0, nv = 0;
+    const bool ride = op_rides(S, f->lat, prec, op);
     VEC(prec, V_BI_P, n, V.p, V.r, V.v, nullptr, nullptr, nullptr, nullptr, nullptr);
     void* y = V.p;
     if (pc) {
@@ -850,8 +872,8 @@ ufg_status run_bicgstab(ufg_solver* S, ufg_field* f, int prec, int op, double to
       y = V.y;
     }
     UFG_TRY(apply_op(S, f, prec, op, y, V.v, 1.0, nullptr, 0.0, V.rhat, false, slot(S, P_SLICE1),
-                     &nsv, S->mom ? OP_BI_ALPHA : -1));
-    if (!S->mom) SCALAR(OP_BI_ALPHA, slot(S, P_SLICE1), nsv, nullptr, 0);
+                     &nsv, ride ? OP_BI_ALPHA : -1));
+    if (!ride) SCALAR(OP_BI_ALPHA, slot(S, P_SLICE1), nsv, nullptr, 0);
     VEC_SCALAR(prec, V_BI_S, n, V.s, V.r, V.v, V.x, y, nullptr, slot(S, P_VEC1), &nv,
                OP_BI_SCHECK);
     void* z = V.s;
@@ -860,8 +882,8 @@ ufg_status run_bicgstab(ufg_solver* S, ufg_field* f, int prec, int op, double to
       z = V.z;
     }
     UFG_TRY(apply_op(S, f, prec, op, z, V.t, 1.0, nullptr, 0.0, V.s, true, slot(S, P_SLICE2),
-                     &nst, S->mom ? OP_BI_OMEGA : -1));
-    if (!S->mom) SCALAR(OP_BI_OMEGA, slot(S, P_SLICE2), nst, nullptr, 0);
+                     &nst, ride ? OP_BI_OMEGA : -1));
+    if (!ride) SCALAR(OP_BI_OMEGA, slot(S, P_SLICE2), nst, nullptr, 0);
     VEC_SCALAR(prec, V_BI_X, n, V.x, z, V.r, V.s, V.t, V.rhat, slot(S, P_VEC2), &nv,
                OP_BI_RCHECK_RHO);
     return UFG_OK;
