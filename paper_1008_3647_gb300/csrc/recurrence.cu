@@ -85,12 +85,18 @@ struct RecArgs {
   double c0, c1;
 };
 
-template <typename R, int ACC, bool OUT, int G = 1>  // ACC = acc_mode; OUT: write out
-__global__ void __launch_bounds__(32 * REC_NCH, sizeof(R) == 4 ? REC_MINB : 5) recurrence_kernel(const RecArgs<R> a) {
+// ML: modes per CTA.  8 for FP64 on a single lattice whose 32-mode CTAs would leave SMs idle (the
+// same arithmetic and 8 chunks; a warp then holds four chunks): FP64 8^3 x 64 runs on 64 SMs' FP64
+// pipes instead of 16 (bicgstab 8^3 x 64 5.28 -> 5.05 ms, with the cheaper scalar steps).  FP32 is
+// bound by load latency and keeps 32 (order-2 series on 16^3 x 256: 71.5 us with 8, 70.0 with 32).
+constexpr int REC_ML_SMALL = 8;
+template <typename R, int ACC, bool OUT, int G, int ML>  // ACC = acc_mode; OUT: write out
+__global__ void __launch_bounds__(ML * REC_NCH, ML < 32 ? 8 : sizeof(R) == 4 ? REC_MINB : 5)
+recurrence_kernel(const RecArgs<R> a) {
   pdl_begin();
-  __shared__ R Es[REC_NCH][32];
-  __shared__ R Ps[REC_NCH][32];
-  __shared__ R Is[REC_NCH][32];
+  __shared__ R Es[REC_NCH][ML];
+  __shared__ R Ps[REC_NCH][ML];
+  __shared__ R Is[REC_NCH][ML];
   const int lane = threadIdx.x;
   const int ch = threadIdx.y;
   long long V = a.V, mode;
@@ -106,7 +112,7 @@ __global__ void __launch_bounds__(32 * REC_NCH, sizeof(R) == 4 ? REC_MINB : 5) r
     done = pr.done;
     mode = (long long)tl.y * 32 + lane;
   } else {
-    mode = (long long)blockIdx.x * 32 + lane;
+    mode = (long long)blockIdx.x * ML + lane;
   }
   if (done != nullptr && a.exec_if >= 0 && *done != a.exec_if) return;
   const bool active = mode < V;
@@ -198,38 +204,36 @@ __global__ void __launch_bounds__(32 * REC_NCH, sizeof(R) == 4 ? REC_MINB : 5) r
   }
 }
 
-template <typename R>
-static cudaError_t rec_launch(const RecArgs<R>& a, unsigned grid, cudaStream_t st) {
-  const dim3 blk(32, REC_NCH);
+template <typename R, int ML>
+static cudaError_t rec_launch_ml(const RecArgs<R>& a, unsigned grid, cudaStream_t st) {
+  const dim3 blk(ML, REC_NCH);
   const bool out = a.out != nullptr;
   if (a.acc_mode != 0 && a.acc == nullptr) return cudaErrorInvalidValue;
+  if (a.acc_mode == 3 && (a.e0 == nullptr || a.e1 == nullptr)) return cudaErrorInvalidValue;
   // FP32: pass 2 in groups, of REC_G_ONE elements where it reads only the input, of REC_G_TWO
   // where it also reads the accumulator or the earlier terms
-  if constexpr (sizeof(R) == 4) {
-    auto go = [&](auto kern) { return launch_k(kern, dim3(grid), blk, 0, st, 1, a); };
-    switch (a.acc_mode * 2 + (out ? 1 : 0)) {
-      case 1: return go(recurrence_kernel<R, 0, true, REC_G_ONE>);
-      case 2: return go(recurrence_kernel<R, 1, false, REC_G_ONE>);
-      case 3: return go(recurrence_kernel<R, 1, true, REC_G_ONE>);
-      case 4: return go(recurrence_kernel<R, 2, false, REC_G_TWO>);
-      case 5: return go(recurrence_kernel<R, 2, true, REC_G_TWO>);
-      case 6:
-        if (a.e0 == nullptr || a.e1 == nullptr) return cudaErrorInvalidValue;
-        return go(recurrence_kernel<R, 3, false, REC_G_TWO>);
-    }
-    return cudaErrorInvalidValue;
-  }
+  constexpr int G1 = sizeof(R) == 4 ? REC_G_ONE : 1, G2 = sizeof(R) == 4 ? REC_G_TWO : 1;
+  auto go = [&](auto kern) { return launch_k(kern, dim3(grid), blk, 0, st, 1, a); };
   switch (a.acc_mode * 2 + (out ? 1 : 0)) {
-    case 1: return launch_k(recurrence_kernel<R, 0, true>, dim3(grid), blk, 0, st, 1, a);
-    case 2: return launch_k(recurrence_kernel<R, 1, false>, dim3(grid), blk, 0, st, 1, a);
-    case 3: return launch_k(recurrence_kernel<R, 1, true>, dim3(grid), blk, 0, st, 1, a);
-    case 4: return launch_k(recurrence_kernel<R, 2, false>, dim3(grid), blk, 0, st, 1, a);
-    case 5: return launch_k(recurrence_kernel<R, 2, true>, dim3(grid), blk, 0, st, 1, a);
-    case 6:
-      if (a.e0 == nullptr || a.e1 == nullptr) return cudaErrorInvalidValue;
-      return launch_k(recurrence_kernel<R, 3, false>, dim3(grid), blk, 0, st, 1, a);
+    case 1: return go(recurrence_kernel<R, 0, true, G1, ML>);
+    case 2: return go(recurrence_kernel<R, 1, false, G1, ML>);
+    case 3: return go(recurrence_kernel<R, 1, true, G1, ML>);
+    case 4: return go(recurrence_kernel<R, 2, false, G2, ML>);
+    case 5: return go(recurrence_kernel<R, 2, true, G2, ML>);
+    case 6: return go(recurrence_kernel<R, 3, false, G2, ML>);
   }
   return cudaErrorInvalidValue;  // nothing to write
+}
+// V modes of one lattice (batched: V = 0, `grid` 32-mode tiles)
+template <typename R>
+static cudaError_t rec_launch(const RecArgs<R>& a, unsigned grid, cudaStream_t st) {
+  if (a.tiles != nullptr) return rec_launch_ml<R, 32>(a, grid, st);
+  if constexpr (sizeof(R) == 8) {
+    if (a.V < 32 * 152)
+      return rec_launch_ml<R, REC_ML_SMALL>(
+          a, (unsigned)((a.V + REC_ML_SMALL - 1) / REC_ML_SMALL), st);
+  }
+  return rec_launch_ml<R, 32>(a, (unsigned)((a.V + 31) / 32), st);
 }
 
 cudaError_t launch_recurrence(int prec, const void* in, void* out, const void* bk, long long V,
@@ -237,17 +241,16 @@ cudaError_t launch_recurrence(int prec, const void* in, void* out, const void* b
                               double acc_coef, int acc_mode, const int* done, cudaStream_t st,
                               const void* e0, const void* e1, double c0, double c1) {
   if (V <= 0 || ntau <= 0) return cudaErrorInvalidValue;
-  const unsigned grid = (unsigned)((V + 31) / 32);
   if (prec == 0) {
     RecArgs<double> a{(const double*)in, (double*)out, (const double*)bk, V, ntau, transpose,
                       out_scale, (double*)acc, acc_coef, acc_mode, done, 0, nullptr, nullptr,
                       (const double*)e0, (const double*)e1, c0, c1};
-    return rec_launch(a, grid, st);
+    return rec_launch(a, 0, st);
   }
   RecArgs<float> a{(const float*)in, (float*)out, (const float*)bk, V, ntau, transpose, out_scale,
                    (float*)acc, acc_coef, acc_mode, done, 0, nullptr, nullptr,
                    (const float*)e0, (const float*)e1, c0, c1};
-  return rec_launch(a, grid, st);
+  return rec_launch(a, 0, st);
 }
 
 cudaError_t launch_recurrence_batch(int prec, const void* in, void* out, const void* bk,
