@@ -581,8 +581,9 @@ def run_ufg(args, rank, world, local_rank):
 def apply_roofline(ufg, torch, dev, stream, hbm, peak_src):
     """Times the fused M and M^T applies on 32^3 x 512 (16.8M sites; x, w and y exceed L2
     together) with CUDA events on the launching stream; algorithmic bytes = read x + read w +
-    write y.  FP64 is bound by the FP64 pipe on this part: its fraction is taken against the FMA
-    throughput measured here by the library (ufg_measure_fma_rate)."""
+    write y.  The FP64 line passes run in fixed point on the integer pipe: their FP64-equivalent
+    rate is set beside the FMA throughput of the FP64 pipe measured here by the library
+    (ufg_measure_fma_rate), which it may exceed."""
     from paper_1008_3647_gb300.inputs import field_and_source
     nx, nt = 32, 512
     lat = ufg.Lattice(nx, nt)
@@ -623,7 +624,7 @@ def apply_roofline(ufg, torch, dev, stream, hbm, peak_src):
     f64 = out["fp64"]
     peak64 = ufg.ufg_measure_fma_rate(ufg.UFG_FP64)
     ach64 = flops_site * lat.ntau * nx ** 3 / (f64["us_per_launch"] * 1e-6) / 1e12
-    f64["alu"] = {"bound": "alu (FP64 pipe)", "achieved": ach64, "peak": peak64,
+    f64["alu"] = {"bound": "alu (integer pipe; FP64-equivalent rate over the FP64 pipe's)", "achieved": ach64, "peak": peak64,
                   "unit": "TFLOP/s", "frac": ach64 / peak64, "flops_per_site": flops_site,
                   "peak_source": "measured in this run (ufg_measure_fma_rate, FP64 FMA chains)"}
     # Q = M^T M: on 32^3 x 512 as M then M^T (24 B/site: x, w, y written and read, q), on
