@@ -265,22 +265,22 @@ static void pack(const std::vector<double>& flat, std::vector<unsigned char>& ou
 }
 
 template <int N>
-static bool pack_fix_n(const double* flat, std::vector<unsigned char>& out) {
+static bool pack_fix_n(const double* flat, double norm, std::vector<unsigned char>& out) {
   LineCoefFix<N> t;
-  if (!fix_table<N>(flat, &t)) return false;
+  if (!fix_table<N>(flat, norm, &t)) return false;
   out.resize(sizeof(t));
   std::memcpy(out.data(), &t, sizeof(t));
   return true;
 }
-static bool pack_fix(int N, const double* flat, std::vector<unsigned char>& out) {
+static bool pack_fix(int N, const double* flat, double norm, std::vector<unsigned char>& out) {
   switch (N) {
-    case 4: return pack_fix_n<4>(flat, out);
-    case 6: return pack_fix_n<6>(flat, out);
-    case 8: return pack_fix_n<8>(flat, out);
-    case 10: return pack_fix_n<10>(flat, out);
-    case 12: return pack_fix_n<12>(flat, out);
-    case 16: return pack_fix_n<16>(flat, out);
-    case 32: return pack_fix_n<32>(flat, out);
+    case 4: return pack_fix_n<4>(flat, norm, out);
+    case 6: return pack_fix_n<6>(flat, norm, out);
+    case 8: return pack_fix_n<8>(flat, norm, out);
+    case 10: return pack_fix_n<10>(flat, norm, out);
+    case 12: return pack_fix_n<12>(flat, norm, out);
+    case 16: return pack_fix_n<16>(flat, norm, out);
+    case 32: return pack_fix_n<32>(flat, norm, out);
   }
   return false;
 }
@@ -318,7 +318,13 @@ static ufg_status build_tables(ufg_lattice* L) {
       return UFG_INTERNAL;
     }
     pack<double>(flat, L->coef[sp.fam][0]);
-    if (!pack_fix(N, flat.data(), L->coef_fix[sp.fam])) {
+    double norm = 0.0;
+    for (int i = 0; i < N; ++i) {
+      double row = 0.0;
+      for (int j = 0; j < N; ++j) row += std::fabs((*sp.A)[(size_t)i * N + j]);
+      norm = std::fmax(norm, row);
+    }
+    if (!pack_fix(N, flat.data(), norm, L->coef_fix[sp.fam])) {
       set_error("line operator of family %d exceeds the fixed-point range", sp.fam);
       return UFG_INTERNAL;
     }

@@ -90,7 +90,9 @@ bool kinetic_coef(double tau, int dispersion, LineCoefFix<N>* c) {
     for (int j = 1; j < H; ++j) co[(i - 1) * (H - 1) + (j - 1)] = 0.5 * (t(i - j) - t(i + j));
   if (!line_coef_flat(N, ce, co, false, false, flat) || (int)flat.size() != LineShape<N>::NC)
     return false;
-  return fix_table<N>(flat.data(), c);
+  double norm = 0.0;  // every row of T holds the same entries
+  for (int i = 0; i < N; ++i) norm += std::fabs(T[i]);
+  return fix_table<N>(flat.data(), norm, c);
 }
 
 template <int N>

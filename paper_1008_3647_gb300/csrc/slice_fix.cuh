@@ -1,13 +1,14 @@
-// FP64 slice kernels on the integer pipe (fix_ops.cuh): the line passes of every FP64 apply,
-// transform and fused momentum-space operator on 3-D lattices.
+// FP64 slice kernels on the integer pipe (fix_ops.cuh): the line passes of the FP64 applies,
+// transforms and fused momentum-space operators on 3-D lattices (but for the calls that
+// base_call_fp64, lattice.cu, keeps on the FP64 pipe).
 //
 // A warp owns PW whole z-planes of one output slice, lanes = (plane p, column x), so the y-pass
-// takes its lines straight from global memory (consecutive x: full sectors, no staging), the x-
-// and y-passes exchange through the warp's own planes of shared memory with no CTA barrier, and
-// the warp's lines share one exponent (a tile).  Between passes the slice stays in 64-bit
-// integers; only the z-pass, whose lines cross the warps, aligns the tiles' exponents, and only
-// the epilogue converts back.  For the z-pass lanes = (row r, column x) with PW whole y-rows per
-// warp, so its loads, stores and epilogue operands are consecutive in x as well.
+// takes its lines straight from global memory (consecutive x: full sectors, no staging), and the
+// x- and y-passes exchange through the warp's own planes of shared memory with no CTA barrier.
+// Between passes the slice stays in 64-bit integers; every line carries an exponent of its own,
+// left beside its values for the lines that cross it (FixExps), and only the epilogue converts
+// back.  For the z-pass lanes = (row r, column x) with PW whole y-rows per warp, so its loads,
+// stores and epilogue operands are consecutive in x as well.
 //
 //   CTA = spc slices x TS threads (TS = 32 per PW planes), one line per thread and pass, no loops
 //   around a pass (the compiler moves the coefficients out of them into registers, 4 KB of
@@ -15,13 +16,12 @@
 //   N = 32: a cluster of 8 CTAs of 128 threads holds one slice, four planes each; the z-pass
 //   reads the other CTAs' planes through distributed shared memory.
 //
-// Bound by the ALU pipe (16^3 x 1024: 56 % busy, FP64 pipe 36 %, 24 warps per SM) and, at N = 32,
-// by instruction fetch (12 warps per SM, straight-line passes of 33 KB).  us per call, FP64-pipe
-// kernels before -> now: M 32^3 x 512 1473 -> 357, 16^3 x 1024 218 -> 42, 16^3 x 256 93 -> 19,
-// 12^3 x 120 32 -> 11; momentum-space M 16^3 x 1024 353 -> 91 (double-float 247).  Tried: one loop
-// over the three passes with the table indexed by the pass (688 us at 32^3, 57 at 16^3: the
-// coefficients come through LDC), the table in shared memory (706, 55: a broadcast moves 4 bytes a
-// cycle).
+// Bound by the ALU pipe (with one exponent per warp, 16^3 x 1024: 56 % busy, FP64 pipe 36 %, 24
+// warps per SM).  us per call, FP64-pipe kernels -> these: M 32^3 x 512 1471 -> 383, 16^3 x 1024
+// 217 -> 44, 16^3 x 256 93 -> 20, 12^3 x 120 35 -> 11; momentum-space M 16^3 x 1024 352 -> 96
+// (double-float 247).  Tried: one loop over the three passes with the table indexed by the pass
+// (688 us at 32^3, 57 at 16^3: the coefficients come through LDC), the table in shared memory (706,
+// 55: a broadcast moves 4 bytes a cycle).
 #pragma once
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
@@ -102,100 +102,83 @@ __device__ __forceinline__ FixPos<N> fix_pos() {
   const int ts = tid - p.s * S::TS;
   p.wl = ts >> 5;
   p.lane = ts & 31;
-  p.lp = p.lane / N;
-  p.lx = p.lane - p.lp * N;
+  p.on = p.lane < S::PW * N;  // the others go along with the first, without writing
+  p.lp = p.on ? p.lane / N : 0;
+  p.lx = p.on ? p.lane - p.lp * N : 0;
   p.line = p.wl * S::PW + p.lp;
-  p.on = p.lane < S::PW * N;
   return p;
 }
 
-// line back to full precision in registers (per warp): the values of lines far below the slice's
-// largest entry gain the bits that the common exponent left unused
+// Exponents (fix_publish) of the lines that the slices of a CTA exchange: of the first pass, read
+// within a plane, and of the second, read across planes.
 template <int N>
-__device__ __forceinline__ void fix_widen(long long (&V)[N], int& E) {
-  unsigned m = 0;
-#pragma unroll
-  for (int i = 0; i < N; ++i) m = fix_mag(m, V[i]);
-  const int sh = fix_renorm(m);
-  if (sh != 0) {
-#pragma unroll
-    for (int i = 0; i < N; ++i) V[i] = fix_shift(V[i], sh);
-    E -= sh;
-  }
-}
+struct FixExps {
+  using S = FixShape<N>;
+  alignas(16) int top1[S::MAXS][S::NPC][N], raw1[S::MAXS][S::NPC][N];  // [plane][x]
+  alignas(16) int top2[S::MAXS][N][S::NPC], raw2[S::MAXS][N][S::NPC];  // [row][plane]
+};
 
-// One pass of a warp's lines: results to dst[i STEP], brought back into range there.
+// One pass of a thread's line: results to dst[i STEP], their exponents to *top and *raw.
 template <int N, bool IN_SPEC, bool OUT_SPEC, int STEP>
-__device__ __forceinline__ void fix_pass(const long long (&V)[N], int& E, const LineCoefFix<N>& cf,
-                                         long long* dst, bool on) {
+__device__ __forceinline__ void fix_pass(const long long (&V)[N], int E, const LineCoefFix<N>& cf,
+                                         long long* dst, int* top, int* raw, bool on) {
   unsigned m = 0;
-  line_op_int<N, IN_SPEC, OUT_SPEC>(V, reinterpret_cast<const int4*>(cf.c),
-                                    [&](int i, long long val) {
-                                      m = fix_mag(m, val);
-                                      if (on) dst[i * STEP] = val;
-                                    });
-  const int sh = fix_renorm(m);
-  if (sh != 0) {
-    if (on)
-#pragma unroll 4
-      for (int i = 0; i < N; ++i) dst[i * STEP] = fix_shift(dst[i * STEP], sh);
-    E -= sh;
-  }
+  line_op_int<N, IN_SPEC, OUT_SPEC>(V, cf, [&](int i, long long val) {
+    m = fix_mag(m, val);
+    if (on) dst[i * STEP] = val;
+  });
+  if (on) fix_publish<N, STEP>(dst, m, E - cf.g, top, raw);
 }
 
 // The line operator along the three axes of a slice.  In: V, the line (line, lx) of the first
-// axis, exponent E of the warp.  With regions [line][i][lx] of padded rows:
+// axis, exponent E.  With regions [line][i][lx] of padded rows:
 //   pass 0  first axis, results i to rows i of the warp's own regions;
 //   pass 1  x: lane (lp, lx) takes row lx of its region, in place;
 //   pass 2  the axis across the regions, for (row `line`, column lx): its input line in V, ready
 //           for line_op_int, exponent E (fix_two returns before it).
 template <int N, bool IN_SPEC, bool OUT_SPEC>
 __device__ __forceinline__ void fix_two(const FixPos<N>& p, bool on, long long (&V)[N], int& E,
-                                        const LineCoefFix<N> (&cf)[3], long long* sm, int* se_cta,
-                                        int rank) {
+                                        const LineCoefFix<N> (&cf)[3], long long* sm,
+                                        FixExps<N>& ex, int rank) {
   namespace cg = cooperative_groups;
   using S = FixShape<N>;
   long long* const mine = sm + p.line * S::PL;
-  fix_pass<N, IN_SPEC, OUT_SPEC, S::P>(V, E, cf[0], mine + p.lx, on);
+  fix_pass<N, IN_SPEC, OUT_SPEC, S::P>(V, E, cf[0], mine + p.lx, &ex.top1[p.s][p.line][p.lx],
+                                       &ex.raw1[p.s][p.line][p.lx], on);
   __syncwarp();
   long long* const row = mine + p.lx * S::P;
-#pragma unroll
-  for (int x = 0; x < N; ++x) V[x] = on ? row[x] : 0;
-  fix_pass<N, IN_SPEC, OUT_SPEC, 1>(V, E, cf[1], row, on);
-  int* const se_mine = se_cta + p.s * S::WPS;
-  if (p.lane == 0) se_mine[p.wl] = E;
-  int se[S::NTILE];
+  {
+    const int *const top = ex.top1[p.s][p.line], *const raw = ex.raw1[p.s][p.line];
+    E = fix_gather<N>([&](int x) -> const int& { return top[x]; },
+                      [&](int x) -> const int& { return raw[x]; },
+                      [&](int x) -> long long& { return row[x]; }, on, V);
+  }
+  fix_pass<N, IN_SPEC, OUT_SPEC, 1>(V, E, cf[1], row, &ex.top2[p.s][p.lx][p.line],
+                                    &ex.raw2[p.s][p.lx][p.line], on);
   if constexpr (S::C > 1) {
+    static_assert(S::NPC == fix_group<N>(), "one group of exponents per CTA");
     cg::this_cluster().sync();
     const int y = rank * S::NPC + p.line;
-#pragma unroll
-    for (int o = 0; o < S::C; ++o) {
-      const int* r = cg::this_cluster().map_shared_rank(se_cta, o);
-#pragma unroll
-      for (int w = 0; w < S::WPS; ++w) se[o * S::WPS + w] = r[w];
-    }
-    E = se[0];
-#pragma unroll
-    for (int i = 1; i < S::NTILE; ++i) E = max(E, se[i]);
-#pragma unroll
-    for (int o = 0; o < S::C; ++o) {
-      const long long* r = cg::this_cluster().map_shared_rank(sm, o) + y * S::P + p.lx;
-#pragma unroll
-      for (int k = 0; k < S::NPC; ++k)
-        V[o * S::NPC + k] = fix_align(r[k * S::PL], E - se[(o * S::NPC + k) / S::PW]);
-    }
+    E = fix_gather<N>(
+        [&](int z) -> const int& {
+          return cg::this_cluster().map_shared_rank(ex.top2[p.s][y], z / S::NPC)[z % S::NPC];
+        },
+        [&](int z) -> const int& {
+          return cg::this_cluster().map_shared_rank(ex.raw2[p.s][y], z / S::NPC)[z % S::NPC];
+        },
+        [&](int z) -> long long& {
+          return cg::this_cluster().map_shared_rank(
+              sm, z / S::NPC)[(z % S::NPC) * S::PL + y * S::P + p.lx];
+        },
+        on, V);
   } else {
     __syncthreads();
-#pragma unroll
-    for (int w = 0; w < S::NTILE; ++w) se[w] = se_mine[w];
-    E = se[0];
-#pragma unroll
-    for (int i = 1; i < S::NTILE; ++i) E = max(E, se[i]);
-    const long long* const col = sm + p.line * S::P + p.lx;
-#pragma unroll
-    for (int i = 0; i < N; ++i) V[i] = on ? fix_align(col[i * S::PL], E - se[i / S::PW]) : 0;
+    long long* const col = sm + p.line * S::P + p.lx;
+    const int *const top = ex.top2[p.s][p.line], *const raw = ex.raw2[p.s][p.line];
+    E = fix_gather<N>([&](int z) -> const int& { return top[z]; },
+                      [&](int z) -> const int& { return raw[z]; },
+                      [&](int z) -> long long& { return col[z * S::PL]; }, on, V);
   }
-  fix_widen<N>(V, E);
 }
 
 // Partial pair of the CTA and the fused scalar step (any number of threads up to 1024).
@@ -275,7 +258,7 @@ slice_fix_kernel(const __grid_constant__ FixArgs<N> A) {
   constexpr bool IN_SPEC = FAM == FAM_INV, OUT_SPEC = FAM == FAM_FWD;
   constexpr int NN = N * N, VOL = N * NN, C = S::C;
   extern __shared__ __align__(16) unsigned char fix_smem[];
-  __shared__ int se_all[S::MAXS * S::WPS];
+  __shared__ FixExps<N> exps;
   __shared__ alignas(8) uint64_t bar2;
   const FixPos<N> p = fix_pos<N>();
   const int unit = blockIdx.x / C;
@@ -306,14 +289,15 @@ slice_fix_kernel(const __grid_constant__ FixArgs<N> A) {
 #pragma unroll
       for (int y = 0; y < N; ++y) v[y] *= on ? __ldg(A.bkpre + m0 + y * N) : 0.0;
     }
-    E = fix_tile<N>(v, V);
+    E = fix_line<N>(v, V);
   }
-  fix_two<N, IN_SPEC, OUT_SPEC>(p, on, V, E, A.cf, sm, se_all, rank);
+  fix_two<N, IN_SPEC, OUT_SPEC>(p, on, V, E, A.cf, sm, exps, rank);
   double acc_dot = 0.0, acc_self = 0.0;
   if (on) {  // last pass and epilogue: sites (z, y, x) of this thread's column
-    const FixOut fo = fix_out<N>(V, E, (A.shift < 0 && u.t_out != 0) ||
-                                           (A.shift > 0 && u.t_out != u.ntau - 1));
-    const double acoef = u.acoef;
+    const FixOut fo = fix_out(E, A.cf[2].g, (A.shift < 0 && u.t_out != 0) ||
+                                                (A.shift > 0 && u.t_out != u.ntau - 1));
+    // fo.post goes into the addition or the scale
+    const double scale = A.id != nullptr ? u.acoef : u.acoef * fo.post;
     const int q = (rank * S::NPC + p.line) * N + p.lx;
     const size_t obase = u.off + (size_t)u.t_out * VOL + q;
     auto site = [&](int z, double o) {
@@ -322,14 +306,15 @@ slice_fix_kernel(const __grid_constant__ FixArgs<N> A) {
         if (A.bkpost != nullptr) o *= A.bkpost[z * NN + q];
         if (A.post != nullptr) o *= A.post[g];
         if (A.post2 != nullptr) o *= A.post2[g];
-        if (A.id != nullptr) o += A.id[g];
-        o *= acoef;
+        if (A.id != nullptr) o = fmadd(o, fo.post, A.id[g]);
+        o *= scale;
         if (A.U != nullptr) o = fmadd(A.bU, A.U[g], o);
         if (A.V != nullptr) o = fmadd(A.cV, A.V[g], o);
       } else {  // unit scale (fix_launch_fam)
         if constexpr ((EPI & E_BK) != 0) o *= __ldg(A.bkpost + z * NN + q);
         if constexpr ((EPI & E_POST) != 0) o *= __ldg(A.post + g);
-        if constexpr ((EPI & E_ID) != 0) o += __ldg(A.id + g);
+        if constexpr ((EPI & E_ID) != 0) o = fmadd(o, fo.post, __ldg(A.id + g));
+        else o *= fo.post;
       }
       A.out[g] = o;
       if constexpr ((EPI & E_DOT) != 0) {
@@ -338,8 +323,7 @@ slice_fix_kernel(const __grid_constant__ FixArgs<N> A) {
       }
     };
     line_op_int<N, IN_SPEC, OUT_SPEC>(
-        V, reinterpret_cast<const int4*>(A.cf[2].c),
-        [&](int z, long long iv) { site(z, fix_get(fo, iv)); });
+        V, A.cf[2], [&](int z, long long iv) { site(z, fix_get(fo, iv)); });
   }
   if ((EPI & E_DOT) != 0 && (A.want_dotP || A.want_self))
     fix_partials(acc_dot, acc_self, A.partials, A.fop, A.tiles, unit, A.probs, A.scs, A.counters,
@@ -386,7 +370,7 @@ slice_fix_m1w_kernel(const __grid_constant__ FixM1wArgs<N> A) {
   static_assert(S::C == 1, "one CTA holds whole slices");
   constexpr int NN = N * N, VOL = N * NN;
   extern __shared__ __align__(16) unsigned char fix_smem[];
-  __shared__ int se_all[S::MAXS * S::WPS];
+  __shared__ FixExps<N> exps;
   __shared__ alignas(8) uint64_t bar2;
   const FixPos<N> p = fix_pos<N>();
   const int unit = blockIdx.x;
@@ -411,31 +395,30 @@ slice_fix_m1w_kernel(const __grid_constant__ FixM1wArgs<N> A) {
 #pragma unroll
       for (int y = 0; y < N; ++y) v[y] *= on ? __ldg(A.bk + m0 + y * N) : 0.0;
     }
-    E = fix_tile<N>(v, V);
+    E = fix_line<N>(v, V);
   }
-  fix_two<N, true, false>(p, on, V, E, A.ci, sm, se_all, 0);
+  fix_two<N, true, false>(p, on, V, E, A.ci, sm, exps, 0);
   {  // last inverse pass, site multiplier on the column (row `line`, x)
     double v[N];
-    const FixOut fo = fix_out<N>(V, E, neg);
+    const FixOut fo = fix_out(E, A.ci[2].g, neg);
     const double* gs = A.site + u.off + (size_t)t_s * VOL + p.line * N + p.lx;
-    line_op_int<N, true, false>(
-        V, reinterpret_cast<const int4*>(A.ci[2].c), [&](int z, long long iv) {
-          v[z] = on ? __ldg(gs + z * NN) * fix_get(fo, iv) : 0.0;
-        });
-    E = fix_tile<N>(v, V);
+    line_op_int<N, true, false>(V, A.ci[2], [&](int z, long long iv) {
+      v[z] = on ? __ldg(gs + z * NN) * fix_get(fo, iv) : 0.0;
+    });
+    E = fix_line<N>(v, V) + fo.shift;
   }
   __syncthreads();  // every column has been read
-  fix_two<N, false, true>(p, on, V, E, A.cf, sm, se_all, 0);
+  fix_two<N, false, true>(p, on, V, E, A.cf, sm, exps, 0);
   double acc_dot = 0.0, acc_self = 0.0;
   if (on) {  // last forward pass and epilogue: modes (plane, y, x)
-    const FixOut fo = fix_out<N>(V, E);
-    const double acoef = u.acoef, fs = A.full_scale;
+    const FixOut fo = fix_out(E, A.cf[2].g);
+    const double acoef = u.acoef * fo.post, fs = A.full_scale;
     const size_t so = u.off + (size_t)u.t_out * VOL;
     auto mode = [&](int y, double o) {
       const int g = m0 + y * N;
       if constexpr (DIR == 0) o *= __ldg(A.bk + g);
       if constexpr (FULL) {  // acoef = 1 (fix_m1w_launch)
-        o += __ldg(A.in + so + g);
+        o = fmadd(o, fo.post, __ldg(A.in + so + g));
         if (A.U != nullptr) o = fmadd(fs, o, A.bU * A.U[so + g]);  // U may be out
       } else {
         o *= acoef;
@@ -446,7 +429,7 @@ slice_fix_m1w_kernel(const __grid_constant__ FixM1wArgs<N> A) {
         if (A.want_self) acc_self = fmadd(o, o, acc_self);
       }
     };
-    line_op_int<N, false, true>(V, reinterpret_cast<const int4*>(A.cf[2].c),
+    line_op_int<N, false, true>(V, A.cf[2],
                                 [&](int y, long long iv) { mode(y, fix_get(fo, iv)); });
   }
   if constexpr (FULL) {
