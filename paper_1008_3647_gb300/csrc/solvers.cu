@@ -45,7 +45,7 @@ struct ufg_solver {
   int pc_kind = UFG_PC_NONE;
   ufg_pc_params pc = {};
   VecSet vs[2];
-  bool fp64_pipe = false;   // inside a mixed solve (kin_call)
+  bool fp64_pipe = false;   // inside a mixed solve (PipeScope, kin_call)
   double* x64 = nullptr;    // FP64 solution accumulator (outer loops, host staging)
   double* b64 = nullptr;    // FP64 right-hand side staging
   double* r64 = nullptr;    // FP64 residual (outer loops, true residual)
@@ -1115,11 +1115,6 @@ bool momentum_basis(const ufg_solver* S, const ufg_field* f, int op, const ufg_p
 // solve, x = F^T x^.
 ufg_status solve_system(ufg_solver* S, ufg_field* f, int op, const double* rhs, double* x64,
                         bool x0, double tol, const ufg_params* p, SolveOut* out) {
-  struct Pipe {  // the FP64 residuals of a mixed solve (kin_call)
-    ufg_solver* S;
-    Pipe(ufg_solver* s, bool on) : S(s) { S->fp64_pipe = on; }
-    ~Pipe() { S->fp64_pipe = false; }
-  } pipe(S, p->precision == UFG_MIXED);
   if (!momentum_basis(S, f, op, p)) return solve_in_basis(S, f, op, rhs, x64, x0, tol, p, out);
   UFG_TRY(fourier64(S, f, rhs, S->mb64, false));
   if (x0) UFG_TRY(fourier64(S, f, x64, S->mx64, false));
@@ -1150,6 +1145,14 @@ struct CallGuard {  // orders the solver stream after the caller's stream and ba
     cudaEventRecord(S->ev, S->st);
     cudaStreamWaitEvent(user, S->ev, 0);
   }
+};
+
+// The FP64 operator of a mixed solve (kin_call), for the whole call: the residual that the call
+// returns and judges is the one its outer loop stopped on.
+struct PipeScope {
+  ufg_solver* S;
+  PipeScope(ufg_solver* s, const ufg_params* p) : S(s) { S->fp64_pipe = p->precision == UFG_MIXED; }
+  ~PipeScope() { S->fp64_pipe = false; }
 };
 
 double paper_mv(const ufg_solver* S, int iters, bool bicg) {
@@ -1467,6 +1470,7 @@ ufg_status ufg_solve_cg_normal(ufg_solver* S, ufg_field* f, const double* b, dou
   }
   const auto t0 = std::chrono::steady_clock::now();
   CallGuard g(S, as_stream(stream));
+  PipeScope pipe(S, p);
   S->counts = Counts();
   const double* bd = nullptr;
   double* xd = nullptr;
@@ -1512,6 +1516,7 @@ ufg_status ufg_solve_bicgstab_two_step(ufg_solver* S, ufg_field* f, const double
   }
   const auto t0 = std::chrono::steady_clock::now();
   CallGuard g(S, as_stream(stream));
+  PipeScope pipe(S, p);
   S->counts = Counts();
   const double* bd = nullptr;
   double* xd = nullptr;
@@ -1529,12 +1534,6 @@ ufg_status ufg_solve_bicgstab_two_step(ufg_solver* S, ufg_field* f, const double
     // one defect-correction round on the composite residual: x += two_step(b - Q x)
     ++extra;
     const size_t bytes = (size_t)S->lat->S * sizeof(double);
-    if (p->precision == UFG_MIXED && S->lat->nx == 32) {  // its right-hand side, see kin_call
-      S->fp64_pipe = true;
-      const ufg_status rs = residual64(S, f, OPK_Q, xd, bd, S->r64, &rn);
-      S->fp64_pipe = false;
-      UFG_TRY(rs);
-    }
     UFG_CUDA(cudaMemcpyAsync(S->rc64, S->r64, bytes, cudaMemcpyDeviceToDevice, S->st));
     UFG_CUDA(cudaMemcpyAsync(S->xs64, xd, bytes, cudaMemcpyDeviceToDevice, S->st));
     SolveOut c1, c2;
