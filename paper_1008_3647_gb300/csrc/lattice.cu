@@ -850,7 +850,12 @@ extern "C" ufg_status ufg_lattice_autotune(ufg_lattice* L, void* stream) {
     char key[160];
     std::snprintf(key, sizeof(key), "%s %d %d %d", device_name().c_str(), N, L->ntau, prec);
     int C = 0, spc = 0;
+    const int most = prec == 0 ? fix_max_slices(N) : 8;  // FP64: only the slices per CTA vary
     if (lookup(key, &C, &spc)) {
+      if (prec == 0) {  // (files may hold shapes of other kernels)
+        L->spc[0] = std::max(1, std::min(spc, most));
+        continue;
+      }
       L->use_tma[prec] = C == 0;
       if (C > 0) {
         L->C[prec] = C;
@@ -859,17 +864,17 @@ extern "C" ufg_status ufg_lattice_autotune(ufg_lattice* L, void* stream) {
       continue;
     }
     std::vector<std::pair<int, int>> cand;
-    cand.emplace_back(0, 1);  // (0, 1): the TMA-staged kernel (where it applies)
+    if (prec == 1) cand.emplace_back(0, 1);  // (0, 1): the TMA-staged kernel (where it applies)
     const size_t es = prec ? 4 : 8;
     const int cs[] = {1, 2, 4};
     for (int c : cs) {
-      if (c > 1 && (N < 16 || prec == 0)) continue;  // FP64: only the slices per CTA vary
+      if (c > 1 && (N < 16 || prec == 0)) continue;
       if (N % c) continue;
-      for (int s = 1; s <= 8; s *= 2) {
+      for (int s = 1; s <= most; s *= 2) {
         const size_t smem = (size_t)s * (N / c) * N * (N + 1) * es;
-        if (smem > 200 * 1024) continue;
+        if (prec == 1 && smem > 200 * 1024) continue;
         if (s > 1 && (L->ntau + s - 1) / s * c < 152) continue;  // keep at least one wave
-        cand.emplace_back(c, s);
+        cand.emplace_back(prec == 0 ? 0 : c, s);
       }
     }
     if (cand.empty()) continue;
@@ -884,8 +889,9 @@ extern "C" ufg_status ufg_lattice_autotune(ufg_lattice* L, void* stream) {
       set_error("autotune: temporary allocation failed");
       return UFG_OOM;
     }
-    cudaMemsetAsync(x, 0, n * es, st);
-    cudaMemsetAsync(w, 0, n * es, st);
+    // constants: lines of zeros take a path of their own in the fixed-point kernels
+    cudaMemsetAsync(x, 0x3f, n * es, st);
+    cudaMemsetAsync(w, 0x3f, n * es, st);
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -895,7 +901,7 @@ extern "C" ufg_status ufg_lattice_autotune(ufg_lattice* L, void* stream) {
       SliceCall c = base_call(L, FAM_KIN, prec);
       c.allow_tma = cd.first == 0;
       c.C = cd.first == 0 ? L->C[prec] : cd.first;
-      c.spc = cd.first == 0 ? L->spc[prec] : cd.second;
+      c.spc = cd.first == 0 && prec == 1 ? L->spc[prec] : cd.second;
       c.in = x;
       c.pre = w;
       c.id = x;
@@ -925,7 +931,9 @@ extern "C" ufg_status ufg_lattice_autotune(ufg_lattice* L, void* stream) {
     cudaFree(x);
     cudaFree(y);
     cudaFree(w);
-    if (bestc.first == 0) {
+    if (prec == 0) {
+      L->spc[0] = bestc.second;
+    } else if (bestc.first == 0) {
       L->use_tma[prec] = 1;
     } else {
       L->use_tma[prec] = 0;
@@ -943,7 +951,8 @@ extern "C" ufg_status ufg_lattice_launch_shape(const ufg_lattice* L, int precisi
     set_error("launch_shape: bad arguments");
     return UFG_INVALID_ARG;
   }
-  *C = L->use_tma[precision] ? 0 : L->C[precision];
-  *spc = L->spc[precision];
+  const bool fixed = precision == UFG_FP64 && L->dim == 3;  // slice_fix.cuh: the extent sets C
+  *C = fixed || L->use_tma[precision] ? 0 : L->C[precision];
+  *spc = fixed ? std::min(L->spc[0], fix_max_slices(L->nx)) : L->spc[precision];
   return UFG_OK;
 }

@@ -104,6 +104,9 @@ template <int N>
 bool slice_tma_prep_ok(int prec, int allow_tma);
 bool slice_tma_prep_supported(int N, int prec, int allow_tma);
 
+// Time slices per CTA that the FP64 kernels (and the momentum-space kernels below N_x = 16) take:
+// CTAs of up to 256 to 640 threads and 48 KB.
+constexpr int fix_max_slices(int N) { return N <= 6 ? 8 : N <= 10 ? 4 : N == 12 ? 2 : 1; }
 // Runtime dispatch over the supported N (4, 6, 8, 10, 12, 16, 32).
 cudaError_t slice_dispatch(int N, const SliceCall& c, cudaStream_t st);
 bool slice_supported_n(int N);

@@ -52,7 +52,7 @@ struct FixShape {
   static constexpr int SLOT = NPC * PL;
   static constexpr int NTILE = N / PW;   // tiles of one slice
   // slices per CTA that the launchers may ask for (lattice and batch tile shapes)
-  static constexpr int MAXS = N == 4 ? 8 : N == 6 ? 8 : N == 8 ? 4 : N == 10 ? 4 : N == 12 ? 2 : 1;
+  static constexpr int MAXS = fix_max_slices(N);
   static constexpr int NT = TS * MAXS;
 };
 
