@@ -944,13 +944,16 @@ ufg_status build_slice_tiles(Batch& B, const ufg_problem* probs) {
   return UFG_OK;
 }
 
-// Time slices per slice tile, tuned per (N_x, tau) group without a TMA shape (the TMA kernels
-// take one slice per CTA; at N_x = 8 a slice is two whole warps).  Each candidate (1, 2, 4, 8
-// slices within 48 KB of FP64 shared memory and the group's longest N_tau) is timed on the
-// batch's own arenas with the FP32 momentum-space M, where mixed solves spend their time, on
-// zeroed operands, three launches each after one; the fastest is kept (ufg_stats.tile_slices).
+// Time slices per slice tile, tuned per (N_x, tau) group: one at N_x = 16 (the FP32 kernels are
+// TMA-staged, one slice per CTA) and at 8 (a slice is two whole warps).  Each candidate (1, 2, 4, 8
+// slices, at most fix_max_slices and the group's longest N_tau) is timed on the batch's own arenas
+// with the FP32 momentum-space M, where preconditioned mixed solves spend their time, on zeroed
+// operands, three launches each after one; the fastest is kept (ufg_stats.tile_slices).  Other
+// solves take the same tiles: timed instead on the kernel of their own precision and basis, with 8
+// tuned as well, no batch of 6 to 96 problems gained beyond its spread (96 problems in FP64 140.4
+// against 140.4 ms) and unpreconditioned ones lost (32 x 6^3 mixed 738 against 945 ms: their time
+// goes into FP64 kernels after all; 24 x 8^3 mixed 549 against 580).
 ufg_status tune_tiles(Batch& B, const ufg_problem* probs) {
-  auto tma_shape = [](int N, int prec) { return prec ? (N == 16 || N == 32) : (N == 8 || N == 16); };
   bool changed = false, zeroed = false;
   cudaEvent_t e0, e1;
   UFG_CUDA(cudaEventCreate(&e0));
@@ -958,13 +961,10 @@ ufg_status tune_tiles(Batch& B, const ufg_problem* probs) {
   ufg_status result = UFG_OK;
   for (auto& g : B.groups) {
     const int N = g.lat->nx;
-    if (tma_shape(N, 0) || tma_shape(N, 1)) continue;
+    if (N == 8 || N == 16) continue;
     std::vector<int> cand;
-    for (int spc : {1, 2, 4, 8}) {
-      const size_t smem = (size_t)spc * N * (N + 1) * N * sizeof(double);
-      if (spc > 1 && (smem > 48 * 1024 || spc > g.max_ntau)) break;
+    for (int spc = 1; spc <= fix_max_slices(N) && (spc == 1 || spc <= g.max_ntau); spc *= 2)
       cand.push_back(spc);
-    }
     if (cand.size() < 2) continue;
     if (!zeroed) {
       if (cudaMemsetAsync(B.ar[1].x, 0, (size_t)B.S * sizeof(float), B.st) != cudaSuccess ||
