@@ -17,6 +17,17 @@ bool slice_m1w_supported(int N, int prec) {
   return N < 32 && slice_supported_n(N);
 }
 
+int sm_count() {
+  static const int n = [] {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0)
+      v = 152;
+    return v;
+  }();
+  return n;
+}
+
 bool slice_q_supported(int N, int prec, int ntau, int dim) {
   static int env = -1;
   if (env < 0) {
@@ -28,15 +39,7 @@ bool slice_q_supported(int N, int prec, int ntau, int dim) {
   // one CTA per output slice with three kinetic stages: ahead of the two launches of M and M^T
   // while their slices fill at most about two CTAs per SM (16^3 x 256: 10.6 against 13.4 us);
   // behind them on longer lattices (16^3 x 1024: 23.0 against 19.1 us)
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0)
-      v = 152;
-    sms = v;
-  }
-  return ntau <= 2 * sms;
+  return ntau <= 2 * sm_count();
 }
 
 bool slice_tma_prep_supported(int N, int prec, int allow_tma) {

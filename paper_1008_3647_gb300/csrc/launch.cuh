@@ -21,6 +21,8 @@ struct PdlScope {
   PdlScope& operator=(const PdlScope&) = delete;
 };
 
+int sm_count();  // SMs of the device
+
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");

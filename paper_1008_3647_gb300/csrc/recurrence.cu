@@ -229,7 +229,7 @@ template <typename R>
 static cudaError_t rec_launch(const RecArgs<R>& a, unsigned grid, cudaStream_t st) {
   if (a.tiles != nullptr) return rec_launch_ml<R, 32>(a, grid, st);
   if constexpr (sizeof(R) == 8) {
-    if (a.V < 32 * 152)
+    if (a.V < 32 * sm_count())
       return rec_launch_ml<R, REC_ML_SMALL>(
           a, (unsigned)((a.V + REC_ML_SMALL - 1) / REC_ML_SMALL), st);
   }
