@@ -186,9 +186,11 @@ static __device__ __noinline__ void scalar_update(int op, DevScalars* gsc, const
 // `counter`, left at 0 for the next producer) sums the set in fixed order and applies `op` to
 // that problem's scalars.  Partials reach the summing CTA through thread 0's fence before its
 // count (only thread 0 wrote them, so only it fences).
+// NT: threads of the CTA, 0 where they are not known at compile time (whole warps, at most 1024).
 template <int NT = SCAL_NT>
 static __device__ __forceinline__ void last_block_update(int op, DevScalars* sc, const double* part,
                                                         int i0, int i1, unsigned* counter) {
+  const int nt = NT > 0 ? NT : (int)blockDim.x;
   __shared__ int is_last;
   if (threadIdx.x == 0) {
     __threadfence();
@@ -197,9 +199,9 @@ static __device__ __forceinline__ void last_block_update(int op, DevScalars* sc,
   __syncthreads();
   if (!is_last) return;
   __threadfence();
-  __shared__ double red[NT / 32][2];
+  __shared__ double red[NT > 0 ? NT / 32 : 32][2];
   double s0 = 0.0, s1 = 0.0;
-  for (int i = i0 + (int)threadIdx.x; i < i1; i += NT) {
+  for (int i = i0 + (int)threadIdx.x; i < i1; i += nt) {
     s0 += part[2 * i];
     s1 += part[2 * i + 1];
   }
@@ -208,41 +210,7 @@ static __device__ __forceinline__ void last_block_update(int op, DevScalars* sc,
   __syncthreads();
   if (threadIdx.x == 0) {
     s0 = s1 = 0.0;
-    for (int w = 0; w < NT / 32; ++w) {
-      s0 += red[w][0];
-      s1 += red[w][1];
-    }
-    scalar_update(op, sc, part, s0, s1, nullptr, 0.0, 0.0);
-    *counter = 0u;
-  }
-}
-
-// last_block_update for CTAs of any whole number of warps (the FP64 slice kernels, whose CTA size
-// follows the lattice extent).
-static __device__ __forceinline__ void last_block_update_any(int op, DevScalars* sc,
-                                                            const double* part, int i0, int i1,
-                                                            unsigned* counter) {
-  __shared__ int is_last;
-  __shared__ double red[32][2];
-  const int tid = threadIdx.x, nw = (int)(blockDim.x >> 5);
-  if (tid == 0) {
-    __threadfence();
-    is_last = atomicAdd(counter, 1u) == (unsigned)(i1 - i0 - 1);
-  }
-  __syncthreads();
-  if (!is_last) return;
-  __threadfence();
-  double s0 = 0.0, s1 = 0.0;
-  for (int i = i0 + tid; i < i1; i += (int)blockDim.x) {
-    s0 += part[2 * i];
-    s1 += part[2 * i + 1];
-  }
-  const double v = warp_sum2(s0, s1);
-  if ((tid & 15) == 0) red[tid >> 5][(tid >> 4) & 1] = v;
-  __syncthreads();
-  if (tid == 0) {
-    s0 = s1 = 0.0;
-    for (int w = 0; w < nw; ++w) {
+    for (int w = 0; w < nt / 32; ++w) {
       s0 += red[w][0];
       s1 += red[w][1];
     }

@@ -203,10 +203,10 @@ __device__ __forceinline__ void fix_partials(double pd, double ps, double* parti
   if (fop >= 0) {
     if (tiles != nullptr) {
       const int prob = tiles[unit].prob;
-      last_block_update_any(fop, scs + prob, partials, probs[prob].st0 - part_base,
+      last_block_update<0>(fop, scs + prob, partials, probs[prob].st0 - part_base,
                             probs[prob].st1 - part_base, counters + prob);
     } else {  // one lattice: the grid's last CTA
-      last_block_update_any(fop, scs, partials, 0, (int)gridDim.x, counters);
+      last_block_update<0>(fop, scs, partials, 0, (int)gridDim.x, counters);
     }
   }
 }

@@ -29,16 +29,16 @@
 
 namespace ufg {
 
-template <int N, typename R>
+template <int N>
 struct QArgs {
   CUtensorMap tm_in;  // [rows][N] view of x, box = one slice
   // the kinetic line operator once per pass direction (constant-bank operands, see TmaArgs)
-  LineCoef<N, R> cx, cy, cz;
-  const R* w;  // the potential w = 1 + A sin(sigma) [S]
-  R* out;
-  const R* U;
-  const R* V;
-  const R* dotP;
+  LineCoef<N, float> cx, cy, cz;
+  const float* w;  // the potential w = 1 + A sin(sigma) [S]
+  float* out;
+  const float* U;
+  const float* V;
+  const float* dotP;
   double a, bU, cV;
   double* partials;
   int want_dotP, want_self;
@@ -57,15 +57,15 @@ struct QArgs {
 constexpr int Q_NT = 2 * TMA_NT;
 
 // x-pass in place, row r: times the multiplier row w when MUL
-template <int N, typename R, bool MUL, class CF>
-__device__ __forceinline__ void q_xpass(R* X, int r, const R (&w)[N], const CF& cf) {
-  using G = SwzGeom<N, R>;
-  constexpr int CPR = G::RB / 16, EPC = 16 / (int)sizeof(R);
-  R v[N];
+template <int N, bool MUL, class CF>
+__device__ __forceinline__ void q_xpass(float* X, int r, const float (&w)[N], const CF& cf) {
+  using G = SwzGeom<N, float>;
+  constexpr int CPR = G::RB / 16, EPC = 16 / (int)sizeof(float);
+  float v[N];
 #pragma unroll
   for (int c = 0; c < CPR; ++c) {
     const int o = G::chunk(r, c);
-    R vc[EPC], wc[EPC];
+    float vc[EPC], wc[EPC];
 #pragma unroll
     for (int e = 0; e < EPC; ++e) {
       vc[e] = X[o + e];
@@ -75,25 +75,25 @@ __device__ __forceinline__ void q_xpass(R* X, int r, const R (&w)[N], const CF& 
 #pragma unroll
     for (int e = 0; e < EPC; ++e) v[c * EPC + e] = vc[e];
   }
-  swz_store_row<N, R>(X, r, v, cf, false, false);
+  swz_store_row<N, float>(X, r, v, cf, false, false);
 }
 
 // y-pass in place, column l = (plane, x)
-template <int N, typename R, class CF>
-__device__ __forceinline__ void q_ypass(R* X, int l, const CF& cf) {
-  using G = SwzGeom<N, R>;
+template <int N, class CF>
+__device__ __forceinline__ void q_ypass(float* X, int l, const CF& cf) {
+  using G = SwzGeom<N, float>;
   const int p = l / N, x = l - (l / N) * N;
-  R v[N];
+  float v[N];
 #pragma unroll
   for (int y = 0; y < N; ++y) v[y] = X[G::off(p * N + y, x)];
-  line_op<N, R, false, false>(v, cf, [&](int i, R val) { X[G::off(p * N + i, x)] = val; });
+  line_op<N, float, false, false>(v, cf, [&](int i, float val) { X[G::off(p * N + i, x)] = val; });
 }
 
-template <int N, typename R, bool UV, bool DOT>
+template <int N, bool UV, bool DOT>
 __global__ void __launch_bounds__(Q_NT, 2)
-slice_q_kernel(const __grid_constant__ QArgs<N, R> A) {
+slice_q_kernel(const __grid_constant__ QArgs<N> A) {
   pdl_begin();
-  using G = SwzGeom<N, R>;
+  using G = SwzGeom<N, float>;
   constexpr int NN = N * N;
   constexpr int VOL = N * NN;
   static_assert(NN == TMA_NT, "one row, line and column per thread of a half");
@@ -106,33 +106,33 @@ slice_q_kernel(const __grid_constant__ QArgs<N, R> A) {
   if (A.done != nullptr && A.exec_if >= 0 && *A.done != A.exec_if) return;
   const int tm = t == 0 ? ntau - 1 : t - 1;
   const int tp = t == ntau - 1 ? 0 : t + 1;
-  const R sA = t != 0 ? R(-1) : R(1);          // sm(t)
-  const R sB = tp != 0 ? R(-1) : R(1);         // sm(t+1)
-  const R sC = t != ntau - 1 ? R(-1) : R(1);   // st(t)
+  const float sA = t != 0 ? float(-1) : float(1);          // sm(t)
+  const float sB = tp != 0 ? float(-1) : float(1);         // sm(t+1)
+  const float sC = t != ntau - 1 ? float(-1) : float(1);   // st(t)
   unsigned char* const base = tma_smem + ((1024u - (smem_addr(tma_smem) & 1023u)) & 1023u);
-  R* const X0 = reinterpret_cast<R*>(base);
-  R* const X1 = X0 + VOL;
-  R* const X2 = X1 + VOL;
-  R* const X3 = X2 + VOL;  // x_t again, for stage A's epilogue
+  float* const X0 = reinterpret_cast<float*>(base);
+  float* const X1 = X0 + VOL;
+  float* const X2 = X1 + VOL;
+  float* const X3 = X2 + VOL;  // x_t again, for stage A's epilogue
   if (tid == 0) {
     mbar_init(&bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    mbar_expect_tx(&bar, (uint32_t)(4 * VOL * sizeof(R)));
+    mbar_expect_tx(&bar, (uint32_t)(4 * VOL * sizeof(float)));
     tma_load_rows(X0, &A.tm_in, tm * NN, &bar);
     tma_load_rows(X1, &A.tm_in, t * NN, &bar);
     tma_load_rows(X2, &A.tm_in, tp * NN, &bar);
     tma_load_rows(X3, &A.tm_in, t * NN, &bar);
   }
   // this thread's multiplier row of its first x-pass, while the boxes are in flight
-  const R* const w_tm = A.w + (size_t)tm * VOL;
-  const R* const w_t = A.w + (size_t)t * VOL;
-  R wrow[N];
+  const float* const w_tm = A.w + (size_t)tm * VOL;
+  const float* const w_t = A.w + (size_t)t * VOL;
+  float wrow[N];
   {
-    constexpr int EPC = 16 / (int)sizeof(R);
-    const R* src = (tid >= NN ? w_t + (size_t)(tid - NN) * N : w_tm + (size_t)tid * N);
+    constexpr int EPC = 16 / (int)sizeof(float);
+    const float* src = (tid >= NN ? w_t + (size_t)(tid - NN) * N : w_tm + (size_t)tid * N);
 #pragma unroll
     for (int c = 0; c < N / EPC; ++c) {
-      R w4[EPC];
+      float w4[EPC];
       ld16(src + c * EPC, w4);
 #pragma unroll
       for (int e = 0; e < EPC; ++e) wrow[c * EPC + e] = w4[e];
@@ -145,43 +145,43 @@ slice_q_kernel(const __grid_constant__ QArgs<N, R> A) {
   {
     const bool second = tid >= NN;
     const int l = second ? tid - NN : tid;
-    R* const X = second ? X1 : X0;
-    q_xpass<N, R, true>(X, l, wrow, A.cx);
+    float* const X = second ? X1 : X0;
+    q_xpass<N, true>(X, l, wrow, A.cx);
     __syncthreads();
-    q_ypass<N, R>(X, l, A.cy);
+    q_ypass<N>(X, l, A.cy);
     __syncthreads();
-    const R* const id = second ? X2 : X3;
-    R* const dst = second ? X2 : X0;
-    const R sg = second ? sB : sA;
+    const float* const id = second ? X2 : X3;
+    float* const dst = second ? X2 : X0;
+    const float sg = second ? sB : sA;
     const int y = l / N, x = l - (l / N) * N;
-    R v[N];
+    float v[N];
 #pragma unroll
     for (int z = 0; z < N; ++z) v[z] = X[G::off(z * N + y, x)];
-    line_op<N, R, false, false>(v, A.cz, [&](int zp, R val) {
+    line_op<N, float, false, false>(v, A.cz, [&](int zp, float val) {
       const int o = G::off(zp * N + y, x);
       dst[o] = fmadd(sg, val, id[o]);
     });
   }
   __syncthreads();
   // ---- C: q_t = a (y_t + st(t) w_t T(y_{t+1})) + bU U + cV V ----
-  if (tid < NN) q_xpass<N, R, false>(X2, tid, wrow, A.cx);
+  if (tid < NN) q_xpass<N, false>(X2, tid, wrow, A.cx);
   __syncthreads();
-  if (tid < NN) q_ypass<N, R>(X2, tid, A.cy);
+  if (tid < NN) q_ypass<N>(X2, tid, A.cy);
   __syncthreads();
   const size_t obase0 = (size_t)t * VOL;
-  const R ra = R(A.a), rbU = R(A.bU), rcV = R(A.cV);
-  R acc_dot = R(0), acc_self = R(0);
+  const float ra = float(A.a), rbU = float(A.bU), rcV = float(A.cV);
+  float acc_dot = float(0), acc_self = float(0);
   if (tid < NN) {
     const int q = tid;
     const int y = q / N, x = q - (q / N) * N;
-    R v[N];
+    float v[N];
 #pragma unroll
     for (int z = 0; z < N; ++z) v[z] = X2[G::off(z * N + y, x)];
     const size_t obase = obase0 + q;
-    line_op<N, R, false, false>(v, A.cz, [&](int zp, R val) {
+    line_op<N, float, false, false>(v, A.cz, [&](int zp, float val) {
       const size_t g = obase + (size_t)zp * NN;
       const int o = G::off(zp * N + y, x);
-      R r = ra * fmadd(sC * __ldg(w_t + zp * NN + q), val, X0[o]);
+      float r = ra * fmadd(sC * __ldg(w_t + zp * NN + q), val, X0[o]);
       if constexpr (UV) {
         if (A.U != nullptr) r = fmadd(rbU, __ldg(A.U + g), r);
         if (A.V != nullptr) r = fmadd(rcV, __ldg(A.V + g), r);
@@ -214,30 +214,30 @@ slice_q_kernel(const __grid_constant__ QArgs<N, R> A) {
       A.partials[2 * blockIdx.x] = d;
       A.partials[2 * blockIdx.x + 1] = q2;
     }
-    if (A.fop >= 0) last_block_update_any(A.fop, A.scs, A.partials, 0, (int)gridDim.x, A.counters);
+    if (A.fop >= 0) last_block_update<0>(A.fop, A.scs, A.partials, 0, (int)gridDim.x, A.counters);
   }
 }
 
-template <int N, typename R, bool UV, bool DOT>
+template <int N, bool UV, bool DOT>
 inline cudaError_t q_launch(const SliceCall& c, cudaStream_t st) {
   constexpr int VOL = N * N * N;
-  QArgs<N, R> a;
+  QArgs<N> a;
   std::memset(&a, 0, sizeof(a));
   if (c.in == nullptr || c.pre == nullptr || c.out == nullptr || c.coef == nullptr ||
       c.ntau < 3 || c.tiles != nullptr || (c.want_dotP && c.dotP == nullptr) ||
       ((c.want_dotP || c.want_self) && c.partials == nullptr) ||
       (c.fop >= 0 && (!DOT || c.scs == nullptr || c.counters == nullptr)))
     return cudaErrorInvalidValue;
-  if (encode_rows<R>(&a.tm_in, c.in, (long long)c.ntau * VOL, N, N * N) != cudaSuccess)
+  if (encode_rows<float>(&a.tm_in, c.in, (long long)c.ntau * VOL, N, N * N) != cudaSuccess)
     return cudaErrorNotSupported;
-  a.cx = *reinterpret_cast<const LineCoef<N, R>*>(c.coef);
+  a.cx = *reinterpret_cast<const LineCoef<N, float>*>(c.coef);
   a.cy = a.cx;
   a.cz = a.cx;
-  a.w = static_cast<const R*>(c.pre);
-  a.out = static_cast<R*>(c.out);
-  a.U = static_cast<const R*>(c.U);
-  a.V = static_cast<const R*>(c.V);
-  a.dotP = static_cast<const R*>(c.dotP);
+  a.w = static_cast<const float*>(c.pre);
+  a.out = static_cast<float*>(c.out);
+  a.U = static_cast<const float*>(c.U);
+  a.V = static_cast<const float*>(c.V);
+  a.dotP = static_cast<const float*>(c.dotP);
   a.a = c.a;
   a.bU = c.bU;
   a.cV = c.cV;
@@ -252,8 +252,8 @@ inline cudaError_t q_launch(const SliceCall& c, cudaStream_t st) {
   a.counters = c.counters;
   a.err = c.err;
   a.expire = take_expired_wait(st);
-  const size_t smem = 4 * (size_t)VOL * sizeof(R) + 1024;
-  auto kern = slice_q_kernel<N, R, UV, DOT>;
+  const size_t smem = 4 * (size_t)VOL * sizeof(float) + 1024;
+  auto kern = slice_q_kernel<N, UV, DOT>;
   static int configured = 0;
   if (!configured) {
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -268,19 +268,19 @@ inline cudaError_t q_launch(const SliceCall& c, cudaStream_t st) {
   return launch_k(kern, dim3(c.ntau), dim3(Q_NT), smem, st, 1, a);
 }
 
-template <int N, typename R>
+template <int N>
 inline cudaError_t q_launch_epi(const SliceCall& c, cudaStream_t st) {
   const bool uv = c.U != nullptr || c.V != nullptr;
   const bool dot = c.want_dotP || c.want_self;
-  if (uv) return dot ? q_launch<N, R, true, true>(c, st) : q_launch<N, R, true, false>(c, st);
-  return dot ? q_launch<N, R, false, true>(c, st) : q_launch<N, R, false, false>(c, st);
+  if (uv) return dot ? q_launch<N, true, true>(c, st) : q_launch<N, true, false>(c, st);
+  return dot ? q_launch<N, false, true>(c, st) : q_launch<N, false, false>(c, st);
 }
 
 // The fused Q for FP32 16^3 slices, where the one-CTA TMA boxes hold one slice.
 template <int N>
 cudaError_t slice_q_try(const SliceCall& c, cudaStream_t st) {
   if constexpr (N == 16) {
-    if (c.prec == 1) return q_launch_epi<16, float>(c, st);
+    if (c.prec == 1) return q_launch_epi<16>(c, st);
   }
   return cudaErrorNotSupported;
 }

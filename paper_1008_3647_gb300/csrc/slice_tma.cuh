@@ -95,7 +95,8 @@ struct TmaArgs {
 template <int N, typename R>
 struct SwzGeom {
   static constexpr int RB = N * (int)sizeof(R);
-  static_assert(RB == 64 || RB == 128, "TMA path covers 64- and 128-byte rows");
+  static_assert(sizeof(R) == 4 && (RB == 64 || RB == 128),
+                "the TMA path covers FP32 with 64- and 128-byte rows");
   static constexpr unsigned EPC = 16 / sizeof(R);  // elements per 16-byte chunk
   // swizzle phase of row r: chunk c of the row is stored at chunk c ^ f(r)
   __device__ __forceinline__ static unsigned f(unsigned r) {
@@ -161,12 +162,8 @@ __device__ __forceinline__ void swz_store_row_impl(R* xs, int r, const R (&v)[N]
 #pragma unroll
   for (int c = 0; c < CPR; ++c) {
     R* dst = xs + G::chunk(r, c);
-    if constexpr (EPC == 4) {
-      *reinterpret_cast<float4*>(dst) =
-          make_float4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
-    } else {
-      *reinterpret_cast<double2*>(dst) = make_double2(o[2 * c], o[2 * c + 1]);
-    }
+    *reinterpret_cast<float4*>(dst) =
+        make_float4(o[EPC * c], o[EPC * c + 1], o[EPC * c + 2], o[EPC * c + 3]);
   }
 }
 template <int N, typename R, class CF>
@@ -557,7 +554,7 @@ inline cudaError_t encode_rows(CUtensorMap* tm, const void* base, long long nele
   const int rb = N * (int)sizeof(R);
   const CUtensorMapSwizzle sw = rb == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
   CUresult r = encode(
-      tm, sizeof(R) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2,
+      tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
       const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
       CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
@@ -574,7 +571,7 @@ inline cudaError_t encode_planes(CUtensorMap* tm, const void* base, long long ne
   const cuuint32_t box[3] = {(cuuint32_t)N, (cuuint32_t)box_y, (cuuint32_t)N};
   const cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = encode(
-      tm, sizeof(R) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3,
+      tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3,
       const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
       CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -775,7 +772,7 @@ constexpr bool swz_perm() {
 #ifndef UFG_SWZ_PERM
 #define UFG_SWZ_PERM 1
 #endif
-  return UFG_SWZ_PERM != 0 && N == 16 && sizeof(R) == 4;
+  return UFG_SWZ_PERM != 0 && N == 16;
 }
 // position of row r = p N + y under the permutation
 template <int N, bool PERM>
