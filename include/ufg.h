@@ -246,11 +246,13 @@ double ufg_lattice_coupling(const ufg_lattice* lat);
  * message) if any kernel launched on the lattice since the last check ran out of its wait, else
  * UFG_OK.  The paper has no counterpart (failure reporting of this library). */
 ufg_status ufg_lattice_check(const ufg_lattice* lat, void* stream);
-/* Test hook for the failure path above: the next `launches` TMA-staged FP32 or FP64 N_x = 8, 16
- * slice-kernel launches (in any lattice of the process) each run one extra bounded wait on a barrier whose expected bytes
- * never arrive, so that wait runs out after a few hundred polling rounds and raises the flag
- * exactly as a real timeout would.  The kernel's own copies complete as usual, nothing faults or
- * hangs, and the results stay correct; only the reported status changes.  0 cancels. */
+/* Test hook for the failure path above: the next `launches` slice-kernel launches that are
+ * TMA-staged (FP32 N_x = 16, 32), FP64 or FP32 momentum-space at N_x = 8 or FP64 at 16, in any
+ * lattice of the process, each run one extra bounded wait on a barrier whose expected bytes never
+ * arrive, so that wait runs out after a few hundred polling rounds and raises the flag exactly as
+ * a real timeout would (the last three wait on nothing else).  A kernel's own copies complete as
+ * usual, nothing faults or hangs, and the results stay correct; only the reported status changes.
+ * 0 cancels. */
 void ufg_test_expire_waits(int launches);
 /* Autotuner: times the fused M apply for every compiled launch shape (CTAs per cluster C, time
  * slices per CTA) on this lattice, in FP64 and FP32, and keeps the fastest for all later applies

@@ -12,7 +12,7 @@ namespace ufg {
 
 // PDL for the launches of standalone operator calls (a PdlScope alive on the calling thread),
 // and for every launch with UFG_PDL=1; the solvers' launches go without (measured slower on the
-// batched solve).
+// batched solve) but for the fused Q of apply_op.
 bool pdl_enabled();
 struct PdlScope {
   PdlScope();

@@ -111,17 +111,9 @@ ufg_status run_q(int ntau, double tau, int dispersion, double A, const double* x
   // the shared-memory-staged kernels: they contain no bounded device wait, so nothing can run
   // out and there is no failure flag that would need a device allocation or a read-back here
   c.allow_tma = 0;
-  // launch shape as for a lattice of this size (4-CTA clusters for 32^3 FP64 slices)
-  if (N >= 32) {
-    c.C = 4;
-    c.spc = 1;
-  } else {
-    const size_t slice = (size_t)N * N * (N + 1) * sizeof(double);
-    int spc = 1;
-    while (spc < 8 && slice * (spc * 2) <= 48 * 1024 && ntau / (spc * 2) >= 152) spc *= 2;
-    c.C = 1;
-    c.spc = spc;
-  }
+  // slices per CTA as on a lattice of this size
+  c.spc = 1;
+  while (c.spc * 2 <= fix_max_slices(N) && ntau / (c.spc * 2) >= 152) c.spc *= 2;
   (void)A;
   SliceCall m = c;  // t = M x
   m.in = x;

@@ -66,8 +66,8 @@ struct SliceCall {
   int ntau = 0;
   int dim = 3;                 // lattice dimension: 3, or 1 / 2 (slice_lowd.cuh)
   int shift = 0;               // -1: t_in = t_out - 1, +1: t_in = t_out + 1, 0: t_in = t_out
-  int spc = 1;                 // time slices per CTA (cluster)
-  int C = 1;                   // cluster size (1, 2 or 4; N = 32 only uses 2 or 4)
+  int spc = 1;                 // time slices per CTA (cluster); FP64: at most fix_max_slices
+  int C = 1;                   // cluster size of slice_kernel (1, 2 or 4; N = 32 only 2 or 4)
   int nt = 256;                // threads per CTA (the kernels are written for 256)
   // batched mode: scalar op applied to each problem from the partials by its last CTA
   int fop = -1;                // ScalarOp, -1: none
@@ -83,7 +83,7 @@ struct SliceCall {
   // basis, out = full_scale * M x + bU * U with the partials as the KIN family; pre is then the
   // potential w = 1 + A sin(sigma) and a = 1
   int m1w_full = 0;
-  // FP64 on 32^3 lattices: the line passes on the FP64 pipe (slice_kernel.cuh) instead of the
+  // FP64 kinetic calls on 32^3 lattices: the line passes on the FP64 pipe (slice_kernel.cuh) instead of the
   // integer pipe, with `coef` the FP64 table (base_call_fp64)
   int fp64_pipe = 0;
   double full_scale = 1.0;
@@ -113,7 +113,7 @@ bool slice_supported_n(int N);
 // Whether the fused FAM_M1W kernel exists for (N, precision): every extent whose slice one CTA
 // holds.
 bool slice_m1w_supported(int N, int prec);
-// Whether the fused FAM_Q kernel runs for (N, precision, N_tau): N = 16 (FP32 and FP64),
+// Whether the fused FAM_Q kernel runs for (N, precision, N_tau): FP32 N = 16,
 // 3 <= N_tau <= twice the SM count, TMA enabled and UFG_NO_FUSED_Q unset.
 bool slice_q_supported(int N, int prec, int ntau, int dim = 3);
 

@@ -15,8 +15,8 @@
 // rows of the x-passes come from global memory (16-byte loads), the epilogue's w_t per site.
 // Stages A and B run side by side in the two halves of the CTA, and the multiplier rows are
 // requested before the boxes arrive: back to back 13.3 -> 8.0 us at 16^3 x 256 with programmatic
-// dependent launch, which the solvers use for this kernel (CG + Chebyshev 16, mixed: 195 -> 183 us
-// per iteration of 17 Q; without it the launch gaps hid the gain).  Latency-bound: 256 CTAs on
+// dependent launch, which apply_op uses for this kernel (CG + Chebyshev 16, mixed: 195 -> 183 us per
+// iteration of 17 Q, 9 of them launched that way; without it the launch gaps hid the gain).  Latency-bound: 256 CTAs on
 // 152 SMs, issue 27 %.
 // Built for FP32 16^3 slices; slice_q_supported says where it runs.
 #pragma once
