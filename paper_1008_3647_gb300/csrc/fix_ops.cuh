@@ -19,8 +19,8 @@
 // normal, graded and log-uniform vectors: median, 99th percentile and largest relative error of the
 // entries and the 2-norm as those of line_op, where the tables' rounding dominates).  One exponent
 // per warp (one to four planes) was 8 % faster at N = 16 and 32 and 1.3x at 10 and 12 (M 16^3 x 1024
-// 41 against 45 us, 12^3 x 1024 30 against 39), but left the far entries of a point source 1e-10 off
-// instead of 4e-13 at N = 16.
+// 41 against 45 us, 12^3 x 1024 30 against 39), but left the far entries of a point source 8e-11 off
+// instead of 5e-13 at N = 16.
 #pragma once
 #include <cuda_runtime.h>
 
