@@ -148,3 +148,26 @@ def test_range_of_fp64(ufg, nx, ntau):
     small = x * 2.0 ** -530 * 2.0 ** -530
     ref = ufg.ufg_apply_kinetic(field, small * 2.0 ** 530 * 2.0 ** 530) * 2.0 ** -530 * 2.0 ** -530
     assert float((ufg.ufg_apply_kinetic(field, small) - ref).abs().max() * 2.0 ** 1000) <= 2.0 ** -73
+
+
+@pytest.mark.parametrize("nx,ntau", EXTENTS)
+def test_range_of_the_operators(ufg, nx, ntau):
+    # as above through every epilogue: the identity and the multipliers beside the line passes, and
+    # the momentum-space operator, which leaves fixed point and comes back to it half way
+    rng = np.random.default_rng(nx + 1)
+    shape = (ntau, nx, nx, nx)
+    sigma = torch.from_numpy(rng.uniform(-np.pi, np.pi, shape)).cuda()
+    field = ufg.Field(ufg.Lattice(nx, ntau), sigma)
+    x = torch.from_numpy(rng.uniform(-1, 1, shape)).cuda()
+    fns = [ufg.ufg_apply_M, ufg.ufg_apply_M1, ufg.ufg_apply_M1T, ufg.ufg_fourier,
+           lambda f, v: ufg.ufg_fourier(f, v, inverse=True)]
+    if nx != 32:
+        fns.append(ufg.ufg_apply_Mdag)
+    if nx in (8, 16):
+        fns += [ufg.ufg_apply_M_momentum, lambda f, v: ufg.ufg_apply_M_momentum(f, v, transpose=True)]
+    for fn in fns:
+        y = fn(field, x)
+        # F sums up to N^(3/2) entries of x: 2^1015 leaves it and M finite
+        for k in (-960, 1015):
+            z = fn(field, x * 2.0 ** (k // 2) * 2.0 ** (k - k // 2))
+            assert torch.equal(z * 2.0 ** -(k // 2) * 2.0 ** -(k - k // 2), y), (fn, k)
